@@ -193,7 +193,10 @@ typedef struct sj_result {
                                  FP32 filter's bounding-box prune (padded
                                  d <= 8) removed; batched results report the
                                  scheduled evaluations */
-    int64_t n_rechecked;      /* pairs re-decided by the FP64 direct form */
+    int64_t n_rechecked;      /* pairs the kernel's certified bound left open,
+                                 re-decided by the direct form (behind a
+                                 tensor-core filter in binary32 with a bound of
+                                 its own first, else in binary64) */
     int32_t reruns;           /* reruns after the page pool overflowed */
     int32_t kernel;           /* SJ_KERNEL_* actually used */
     double ms_tile;           /* device time of the distance-tile kernel of the

@@ -476,8 +476,7 @@ static int run_join(sj_index* ix, ResultImpl* ri, int64_t page_pairs, bool dist,
     // deferred-recheck queue: band pairs (and, with distances, every
     // maybe-in pair); pairs past its end are re-decided in place
     const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
-    unsigned long long band_cap = dist ? std::max<unsigned long long>(1ull << 20, ev / 8) : std::max<unsigned long long>(1ull << 20, ev / 64);
-    band_cap = std::min<unsigned long long>(band_cap, ev);
+    const unsigned long long band_cap = queue_entries(ix->kernel, ev, dist);
     Scratch tmp(s);
     int2* band = nullptr;
     SJ_TRY(tmp.alloc(&band, (size_t)band_cap));
@@ -505,8 +504,12 @@ static int run_join(sj_index* ix, ResultImpl* ri, int64_t page_pairs, bool dist,
         else
             st = launch_join_cc(ix, jo, dist ? 1 : 0);
         ix->n_items = all_items;
-        if (st == SJ_OK) SJ_CK(cudaEventRecord(ix->ev_tile[1], s));
+        // (a tensor-core filter's tile time includes the resolution of its
+        // records, which emits the pairs)
+        const bool records = is_tensor_kernel(ix->kernel);
+        if (st == SJ_OK && !records) SJ_CK(cudaEventRecord(ix->ev_tile[1], s));
         if (st == SJ_OK) st = launch_recheck(ix, jo, dist ? 1 : 0);
+        if (st == SJ_OK && records) SJ_CK(cudaEventRecord(ix->ev_tile[1], s));
     }
     unsigned long long c[kCounters] = {};
     if (st == SJ_OK) {
@@ -555,7 +558,7 @@ int sj_self_join_to_host(sj_handle h, int32_t* host_pairs, int64_t host_capacity
     cudaStream_t s = ix->stream;
     const int64_t n_items = ix->n_items;
     const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
-    unsigned long long band_cap = std::min<unsigned long long>(std::max<unsigned long long>(1ull << 20, ev / 64), ev);
+    const unsigned long long band_cap = queue_entries(ix->kernel, ev, false);
     int2* pool[2] = {nullptr, nullptr};
     int2* band = nullptr;
     cudaStream_t cs = nullptr;
@@ -964,8 +967,10 @@ static int batch_join_phase(std::vector<std::unique_ptr<BatchGroup>>& groups, co
         if (st == SJ_OK)
             st = is_tensor_kernel(ix->kernel) ? launch_join_tc(ix, jos[gi], dist ? 1 : 0)
                                               : launch_join_cc(ix, jos[gi], dist ? 1 : 0);
+        const bool records = is_tensor_kernel(ix->kernel);  // (timed with their resolution, as in run_join)
+        if (st == SJ_OK && records) st = launch_recheck(ix, jos[gi], dist ? 1 : 0);
         if (st == SJ_OK && cudaEventRecordWithFlags(ix->ev_tile[1], gs, rec) != cudaSuccess) st = SJ_ERR_CUDA;
-        if (st == SJ_OK) st = launch_recheck(ix, jos[gi], dist ? 1 : 0);
+        if (st == SJ_OK && !records) st = launch_recheck(ix, jos[gi], dist ? 1 : 0);
         ix->stream = keep;
         return st;
     };
@@ -1116,6 +1121,7 @@ int join_batch_impl(const double* const* pts, const int64_t* n, const int32_t* d
             dev_free(g->d_gid, s);
             dev_free(g->d_e2, s);
             dev_free(g->d_r2, s);
+            dev_free(g->d_refine, s);
             dev_free(g->d_inst_of_sorted, s);
             dev_free(g->d_item_inst, s);
         }
@@ -1261,6 +1267,7 @@ int join_batch_impl(const double* const* pts, const int64_t* n, const int32_t* d
             bj.inst_gid = g.d_gid;
             bj.inst_e2 = g.d_e2;
             bj.inst_r2 = g.d_r2;
+            bj.inst_refine = g.d_refine;
             bj.pool = reinterpret_cast<int2*>(pool->block);
             bj.dpool = pool->dblock;
             bj.page_log2 = page_log2;
@@ -1275,8 +1282,7 @@ int join_batch_impl(const double* const* pts, const int64_t* n, const int32_t* d
             Index* ix = &g.ix;
             if (ix->n_items == 0) continue;
             const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
-            unsigned long long band_cap =
-                std::min<unsigned long long>(ev, std::max<unsigned long long>(1ull << 20, dist ? ev / 8 : ev / 64));
+            const unsigned long long band_cap = queue_entries(ix->kernel, ev, dist);
             if ((st = dev_alloc_t(&bands[gi], (size_t)band_cap, s)) != SJ_OK) break;
             jos[gi].band = bands[gi];
             jos[gi].band_cap = band_cap;

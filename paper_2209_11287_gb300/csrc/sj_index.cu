@@ -454,6 +454,12 @@ struct PackParams {
     // rule (the small-d FP32 filter's bounding-box prune)
     double prune_r2 = INFINITY;
     float prune_r2f = INFINITY;
+    // Direct form in binary32, s32 = sum of (y_qk - y_ck)^2: every operation
+    // rounds to 2^-24, so |s32 - s_y| <= 1.01 (dp + 3) 2^-24 s_y (a term that
+    // underflows is off by 2^-149, far below the margin for a radius^2 of
+    // 2^-60 or more); twice that is taken.  s32 > refine_out then means s_y >
+    // S_o, out; s32 < refine_in means s_y < S_i, in.
+    float refine_out = INFINITY, refine_in = -1.f;
 };
 
 __host__ __device__ inline double gamma_n(double u, int k) { return k * u / (1.0 - k * u); }
@@ -538,6 +544,9 @@ void pack_coefficients(double eps, double pbound, double delta, double u_t, int 
     pp->bf_in = up(pp->b_in);
     pp->prune_r2 = so;
     pp->prune_r2f = up(so);
+    const double rel = 2.02 * (dp + 3) * ldexp(1.0, -24);
+    pp->refine_out = so >= ldexp(1.0, -60) ? up(so * (1.0 + rel)) : INFINITY;
+    pp->refine_in = si_r > 0 && si >= ldexp(1.0, -60) ? down(si * (1.0 - rel)) : -1.f;
 }
 
 // The two thresholds of a point with computed norm pc, one fma each, rounded
@@ -1534,6 +1543,8 @@ int build_index(Index* ix, const double* pts) {
     ix->kscale = scale;
     pack_coefficients(ix->eps * scale, pbound * scale * scale, delta * scale, u_t, d, ix->dp, &hp, c1);
     ix->prune_r2 = hp.prune_r2f;
+    ix->refine_out = hp.refine_out;
+    ix->refine_in = hp.refine_in;
 
     // ---- cell keys, sort and packing ----
     SJ_TRY(dev_alloc_t(&ix->perm, (size_t)n, s));
@@ -2165,6 +2176,7 @@ int build_batch_group(BatchGroup* g, const double* const* src_dev_ptrs, const in
     std::vector<double> centre((size_t)K * dp, 0.0);
     std::vector<double> e2((size_t)K);
     std::vector<float> r2((size_t)K);
+    std::vector<float2> refine((size_t)K);
     int shift = 0;
     const bool tensor = is_tensor_kernel(ix->kernel);
     const bool use_f32 = ix->kernel == SJ_KERNEL_FILTER_F32 || tensor;
@@ -2223,6 +2235,7 @@ int build_batch_group(BatchGroup* g, const double* const* src_dev_ptrs, const in
         PackParams pp{};
         pack_coefficients(t.eps * sk, pbk * sk * sk, 1.01 * u_t * rmax * sk, u_t, dp, dp, &pp, c1);
         r2[k] = pp.prune_r2f;
+        refine[k] = make_float2(pp.refine_out, pp.refine_in);
         b.a_out = pp.a_out;
         b.b_out = pp.b_out;
         b.a_in = pp.a_in;
@@ -2244,6 +2257,8 @@ int build_batch_group(BatchGroup* g, const double* const* src_dev_ptrs, const in
     SJ_CK(cudaMemcpyAsync(g->d_e2, e2.data(), K * sizeof(double), cudaMemcpyHostToDevice, s));
     SJ_TRY(dev_alloc_t(&g->d_r2, (size_t)K, s));
     SJ_CK(cudaMemcpyAsync(g->d_r2, r2.data(), K * sizeof(float), cudaMemcpyHostToDevice, s));
+    SJ_TRY(dev_alloc_t(&g->d_refine, (size_t)K, s));
+    SJ_CK(cudaMemcpyAsync(g->d_refine, refine.data(), K * sizeof(float2), cudaMemcpyHostToDevice, s));
     // ---- keys, sort, cells ----
     unsigned long long* keys = nullptr;
     SJ_TRY(tmp.alloc(&keys, (size_t)n));

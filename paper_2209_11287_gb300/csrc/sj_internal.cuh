@@ -141,6 +141,9 @@ struct Index {
     // squared distance of kernel coordinates above it is certified out (the
     // radius of the thresholds, see pack_coefficients)
     float prune_r2 = INFINITY;
+    // as prune_r2, for a squared distance evaluated in binary32 (direct form):
+    // above refine_out certainly out, below refine_in certainly in
+    float refine_out = INFINITY, refine_in = -1.f;
     unsigned long long last_pruned = 0;  // pair evaluations the last join's prune removed
 
     // per-join scratch: counters (item queue, result cursor, recheck count,
@@ -196,6 +199,7 @@ struct BatchGroup {
     int32_t* d_gid = nullptr;
     double* d_e2 = nullptr;
     float* d_r2 = nullptr;          // per instance: the bounding-box prune radius^2
+    float2* d_refine = nullptr;     // per instance: refine_out, refine_in
     int32_t* d_inst_of_sorted = nullptr;
     int32_t* d_item_inst = nullptr;
 };
@@ -210,6 +214,7 @@ struct BatchJoin {
     const double* inst_e2;          // group-local instance -> eps^2
     const float* inst_r2;           // group-local instance -> the small-d FP32 filter's
                                     // bounding-box prune radius^2 (kernel units), or null
+    const float2* inst_refine;      // group-local instance -> refine_out, refine_in
     // output (indexed by instance number)
     int2* pool;                     // n_pages pages of 2^page_log2 pairs
     double* dpool;                  // matching distances, or null
@@ -265,7 +270,27 @@ int build_aux(Index* ix);
 int launch_item_work(Index* ix, long long* work);
 int launch_join_tc(Index* ix, const JoinOut& out, int emit_dist);
 int selftest_bounded_wait(cudaStream_t s);
+// What follows a tile kernel: the recheck of the queued pairs, or of a
+// tensor-core filter the resolution of its records (sj_resolve.cu).
 int launch_recheck(Index* ix, const JoinOut& out, int emit_dist);
+int launch_resolve(Index* ix, const JoinOut& out, int emit_dist);
+// Entries (8 bytes) of the recheck queue of a join of `ev` evaluations.  A
+// tensor-core filter keeps its 16-byte records there, one per candidate and 32
+// query columns with a maybe-in pair: at most ev / 16 of them (records past
+// the queue are dealt with in the tile kernel), at most 2 GB above the pairs'
+// own share.
+inline unsigned long long queue_entries(int kernel, unsigned long long ev, bool dist) {
+    const unsigned long long small = ev / (dist ? 8 : 64), least = 1ull << 20;
+    unsigned long long cap = small;
+    if (is_tensor_kernel(kernel)) {
+        const unsigned long long most = small > (1ull << 28) ? small : 1ull << 28;
+        cap = ev / 8 < most ? ev / 8 : most;
+        if (cap < small) cap = small;
+        return cap > least ? cap : least;  // (room for whole reservations however few the evaluations)
+    }
+    if (cap < least) cap = least;
+    return cap < ev ? cap : ev;
+}
 
 // Split products per dim of a tensor-core filter: BF16x3 keeps 6, BF16x2 and
 // FP16x2 3.

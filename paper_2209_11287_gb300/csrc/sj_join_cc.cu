@@ -87,6 +87,7 @@ static int launch_recheck_dp(Index* ix, const JoinParams& p) {
 }
 
 int launch_recheck(Index* ix, const JoinOut& out, int emit_dist) {
+    if (is_tensor_kernel(ix->kernel)) return launch_resolve(ix, out, emit_dist);
     const JoinParams p = make_join_params(ix, out, emit_dist);
     switch (ix->dp) {
         case 2: return launch_recheck_dp<2>(ix, p);
@@ -132,6 +133,8 @@ JoinParams make_join_params(Index* ix, const JoinOut& out, int emit_dist) {
     p.dbg = out.dbg;
     p.dbg_cap = out.dbg_cap;
     p.prune_r2 = ix->prune_r2;
+    p.refine_out = ix->refine_out;
+    p.refine_in = ix->refine_in;
     return p;
 }
 

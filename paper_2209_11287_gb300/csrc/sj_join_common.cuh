@@ -55,6 +55,7 @@ struct JoinParams {
     // per-instance value from BatchJoin::inst_r2); counters[6] counts the
     // pair evaluations this removes
     float prune_r2;
+    float refine_out, refine_in;  // (Index: the same names; batched: per instance)
 };
 
 // Records one evaluated pair for the filter dump.

@@ -13,25 +13,43 @@
 // accumulator ends as a = -||y_q||^2/2 + y_q . y_c, the quantity every other
 // kernel computes.  Each value is compared with per-candidate thresholds
 // widened for this arithmetic (dropped split products and the tensor core's
-// FP32 accumulation); pairs inside the bound are re-decided in binary64 by
-// k_recheck.
+// FP32 accumulation); what is maybe in goes, with what is certainly in, as
+// records (a candidate against 32 query columns) to k_resolve, which decides
+// the pairs inside the bound and writes the result (sj_resolve.cu).
 //
 // One persistent CTA per SM, warp-specialised:
-//   warp 0      producer: takes work items from the queue, loads the item's
-//               query tile (MMA B, N <= 256 queries, 8-row groups from an
-//               8-aligned start) and streams the candidate tiles (MMA A,
-//               128 rows = 16 groups covering the item's runs) in K-slices
-//               of 64 with bulk copies completing on mbarriers;
+//   warp 0      tiles: takes work items from the queue and cuts the item's
+//               candidate runs into tiles (128 rows = 16 8-row groups), per
+//               tile the rows' metadata and the copies that bring them;
 //   warp 1      MMA issuer (one thread): K/16 MMAs per tile into one of two
 //               TMEM accumulators (128 lanes x N columns), committed to the
 //               stage and accumulator barriers;
-//   warps 2..   epilogue (8 to 16 warps): each thread owns one candidate row
-//               (its TMEM lane) and a share of its N accumulators (2 to 4
-//               warps per lane quarter, interleaved 32-column chunks),
-//               compares them with the
-//               candidate's two thresholds (a max over 32 columns first; hits
-//               are rare), then runs the warp-aggregated emission of the
-//               CUDA-core kernels.
+//   warp 2      copies (one thread): the item's query tile (MMA B, N <= 256
+//               queries, 8-row groups from an 8-aligned start; the next
+//               item's while this one runs, where shared memory allows) and
+//               the candidate tiles (MMA A) in K-slices of 64, bulk copies
+//               completing on mbarriers;
+//   warps 3..   epilogue (16 or 8 warps): each thread owns one candidate row
+//               (its TMEM lane) and a share of its N accumulators (EPI / 4
+//               warps per lane quarter, interleaved 32-column chunks): a max
+//               over the chunk against the row's threshold first (hits are
+//               rare), then column masks of the maybe-in and the certain ones
+//               and a record.
+// What bounds it: at K = 64 the epilogue's instruction issue (57% of the issue
+// slots, about 330 instructions a warp and tile), so it holds only what has to
+// happen while the accumulator is there, and an accumulator is released as
+// soon as its last columns are in registers.  Emitting the pairs here (ids,
+// compaction, pages, recheck queue, by half-empty warps) made every warp wait
+// for that serial code in turn.  Resolving the rows of a tile and its copies
+// used to be one warp's work (about 1,100 cycles a tile, 1,900 with many runs,
+// slower than the MMA's 512); the two halves now overlap.  16 epilogue warps
+// with one chunk in registers each (96 registers) against 8 warps with two
+// (150): 1.99 / 2.34 ms (2^17 x 16-D without an index), 2.84 / 3.14 (500,000 x
+// 16-D mixture), 4.07 / 3.83 (150,000 x 64-D): at K = 208 the MMA binds (the
+// shared-memory reads of its operands, 12 KB per 128 cycles) and more warps
+// only compete with it, so the line lies between K = 112 and 208.  Tile kernel
+// before / now: 2.85 / 1.99 ms, 5.21 / 2.84 ms, and 7.50 / 6.89 ms at 200,000 x
+// 64-D.
 // A symmetric join evaluates only the triangle of each self cell: the self
 // run starts at the item's first query and pairs below the diagonal are
 // masked.  Every wait is bounded; on expiry the CTA stops issuing work,
@@ -46,12 +64,12 @@ namespace sj {
 constexpr int kTcM = 128;             // candidate rows per tile (TMEM lanes)
 constexpr int kTcG = kTcM / 8;        // 8-row groups per tile
 constexpr int kKS = 64;               // K per pipeline slice
-constexpr int kMetaDepth = 4;         // tiles of row metadata in flight
-// Epilogue warps: EPI / 4 per TMEM lane quarter, splitting the columns; as
-// many as shared memory allows next to the query tile (the epilogue's
-// latency is what bounds the tile rate when hits are frequent).
-constexpr int tc_epi(int kp, bool emit) { return kp <= 112 ? 16 : (emit ? 8 : 12); }
-constexpr int tc_threads(int kp, bool emit) { return 64 + 32 * tc_epi(kp, emit); }  // producer, MMA, epilogue
+constexpr int kMetaDepth = 8;         // tiles of row metadata in flight
+// Epilogue warps (EPI / 4 per TMEM lane quarter, splitting the columns) and
+// the 32-column chunks a warp holds at a time.
+constexpr int tc_epi(int kp) { return kp <= 112 ? 16 : 8; }
+constexpr int tc_chunks(int kp) { return kp <= 112 ? 1 : 2; }
+constexpr int tc_threads(int kp) { return 96 + 32 * tc_epi(kp); }  // tile, MMA and copy warps, epilogue
 constexpr long long kTcSpin = 1 << 22;  // bound on barrier polls per wait
 
 struct TcParams {
@@ -68,6 +86,7 @@ struct TcShape {
     static constexpr int SLICES = (KP + kKS - 1) / kKS;
     static constexpr int A_STAGE = kTcM * kKS * 2;  // bytes
     static constexpr int B_BYTES = NMAX * KP * 2;
+    static constexpr int NB = KP <= 112 ? 2 : 1;  // query tiles in flight (as shared memory allows)
 };
 
 // Per-item information shared by the roles (a ring of two).
@@ -79,22 +98,22 @@ struct TcItem {
     int ntiles;        // candidate tiles
 };
 
-// Per-tile row metadata: each 8-row group's first row (-1: none), the run's
-// valid position range and its flag (0 plain, 1 mirror, 2 self triangle).
+// Per-tile row metadata: each 8-row group's first row (-8: none), the run's
+// valid position range and its flag (0 plain, 1 mirror, 2 self triangle); and
+// the copies that bring the tile: rows of consecutive groups of the index.
 struct TcMeta {
-    int32_t g[kTcG];
-    int32_t lo[kTcG];
-    int32_t hi[kTcG];
-    uint8_t fl[kTcG];
+    int4 g[kTcG];       // first row, first and past-the-last valid position, flag
+    int32_t nseg, cnt;  // copies, groups
+    int4 seg[kTcG];     // first group in the tile, groups, first group of the index, -
 };
 
-template <int KP, bool EMIT>
+template <int KP>
 struct TcSmem {
-    static constexpr int EPI = tc_epi(KP, EMIT);
+    static constexpr int EPI = tc_epi(KP);
     static_assert(EPI % 4 == 0, "epilogue warps come in whole warpgroups");
-    static constexpr int MAX_STAGES = 6;
+    static constexpr int MAX_STAGES = 8;
     uint64_t a_full[MAX_STAGES], a_empty[MAX_STAGES];
-    uint64_t b_full, b_empty;
+    uint64_t b_full[2], b_empty[2];
     uint64_t item_full[2], item_empty[2];
     uint64_t meta_full[kMetaDepth], meta_empty[kMetaDepth];
     uint64_t acc_full[2], acc_empty[2];
@@ -102,29 +121,25 @@ struct TcSmem {
     uint32_t tmem;
     int abort;
     TcItem items[2];
-    int32_t qperm[2][256];  // input index of each query-tile row of the items in the ring
     TcMeta meta[kMetaDepth];
-    int32_t rgp[kMaxRuns];  // producer: per run of the item, its first group's number in the item
+    int32_t rgp[kMaxRuns];  // tile warp: per run of the item, its first group's number in the item
     int32_t rlo[kMaxRuns], rhi[kMaxRuns];
     uint8_t rfl[kMaxRuns];
-    int2 stage[EPI][kStage];
-    double sdist[EPI][EMIT ? kStage : 1];
-    uint16_t hits[EPI][32][32];  // per epilogue warp: maybe-in entries of a 32-column chunk, per lane
 };
 
 // Operand stages: as many as fit (up to 6) in the 227 KB of shared memory a
 // CTA may use next to the query tile and the rest.
 constexpr size_t kSmemMax = 232448;
-template <int KP, bool EMIT>
+template <int KP>
 __host__ __device__ constexpr int tc_stages() {
-    const long long left = (long long)kSmemMax - 1024 - TcShape<KP>::B_BYTES - (long long)sizeof(TcSmem<KP, EMIT>);
+    const long long left = (long long)kSmemMax - 1024 - TcShape<KP>::NB * TcShape<KP>::B_BYTES - (long long)sizeof(TcSmem<KP>);
     const long long st = left / TcShape<KP>::A_STAGE;
-    return st > TcSmem<KP, EMIT>::MAX_STAGES ? TcSmem<KP, EMIT>::MAX_STAGES : (int)st;
+    return st > TcSmem<KP>::MAX_STAGES ? TcSmem<KP>::MAX_STAGES : (int)st;
 }
-template <int KP, bool EMIT>
+template <int KP>
 constexpr size_t tc_smem_bytes() {
-    return 1024 /* alignment slack */ + (size_t)TcShape<KP>::B_BYTES +
-           (size_t)tc_stages<KP, EMIT>() * TcShape<KP>::A_STAGE + sizeof(TcSmem<KP, EMIT>);
+    return 1024 /* alignment slack */ + (size_t)TcShape<KP>::NB * TcShape<KP>::B_BYTES +
+           (size_t)tc_stages<KP>() * TcShape<KP>::A_STAGE + sizeof(TcSmem<KP>);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -179,6 +194,10 @@ __device__ __forceinline__ bool bar_wait_n(uint64_t* b, uint32_t parity, volatil
 __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, volatile int* abort) {
     return bar_wait_n(b, parity, abort, kTcSpin);
 }
+// The wait of a whole warp: one answer for all lanes.
+__device__ __forceinline__ bool bar_wait_warp(uint64_t* b, uint32_t parity, volatile int* abort) {
+    return __all_sync(0xffffffffu, bar_wait(b, parity, abort));
+}
 // Bulk copy global -> shared completing on an mbarrier.
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile(
@@ -191,21 +210,16 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-// 16 consecutive TMEM columns of this thread's lane (no wait).
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr));
-}
-
 // Three-input maximum (one instruction on this architecture).
 __device__ __forceinline__ float max3f(float a, float b, float c) {
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
+}
+
+// (mask << 1) | sign bit of v: one funnel shift.
+__device__ __forceinline__ uint32_t push_sign(uint32_t mask, float v) {
+    return __funnelshift_l(__float_as_uint(v), mask, 1);
 }
 
 // 32 consecutive TMEM columns of this thread's lane (no wait).
@@ -221,19 +235,84 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
         : "r"(taddr));
 }
 
+// A record: one candidate against 32 query positions from a first one on, as
+// (maybe-in columns, certain ones, first position, candidate position | kMirrorBit
+// when its pairs are emitted in both orders, the diagonal excepted).  A warp
+// takes room in the queue 64 records at a time with one atomic.
+constexpr int kTcChunk = 64;
+struct TcRecords {
+    unsigned long long base;  // next reserved record
+    int left;                 // reserved records left (warp-uniform)
+};
+
+// A record that found no room: its pairs are decided and written here, one
+// lane each (rare: the queue holds a record for every 16 evaluations).
+__device__ __noinline__ void tc_resolve_here(const JoinParams& P, int4 e) {
+    const int32_t cs = (int32_t)((uint32_t)e.w & ~kMirrorBit);
+    unsigned long long decided = 0;
+    for (uint32_t m = (uint32_t)e.x; m; m &= m - 1u) {
+        const int k = __ffs(m) - 1;
+        const int32_t qs = e.z + k;
+        if (P.emit_dist || !((uint32_t)e.y >> k & 1u)) ++decided;
+        const int li = P.batch ? P.batch->inst_of_sorted[qs] : 0;
+        const double s = direct_sq(P.xs + (int64_t)qs * P.dp, P.xs + (int64_t)cs * P.dp, P.d);
+        if (!(s <= (P.batch ? P.batch->inst_e2[li] : P.e2))) continue;
+        const int nout = e.w < 0 && cs != qs ? 2 : 1;
+        const int32_t qid = P.perm[qs], cid = P.perm[cs];
+        const double dist = P.emit_dist ? sqrt(s) : 0.0;
+        if (P.batch) {
+            const int32_t off = (int32_t)P.batch->inst_off[li];
+            batch_emit_one(P, P.batch->inst_gid[li], nout, qid - off, cid - off, dist);
+        } else {
+            const unsigned long long at = atomicAdd(&P.counters[1], (unsigned long long)nout);
+            for (int u = 0; u < nout; ++u)
+                if (at + u < P.capacity) {
+                    P.out_pairs[at + u] = u == 0 ? make_int2(qid, cid) : make_int2(cid, qid);
+                    if (P.emit_dist) P.out_dist[at + u] = dist;
+                }
+        }
+    }
+    if (decided) atomicAdd(&P.counters[2], decided);
+}
+
+// Warp-collective: the lanes whose record has columns append it.
+__device__ __forceinline__ void tc_record(TcRecords& rec, const JoinParams& P, int lane, int4 e) {
+    const unsigned b = __ballot_sync(0xffffffffu, e.x != 0);
+    const int n = __popc(b), r = __popc(b & ((1u << lane) - 1u));
+    unsigned long long pos = rec.base + (unsigned long long)r;
+    if (n <= rec.left) {
+        rec.base += (unsigned long long)n;
+        rec.left -= n;
+    } else {  // the rest of this reservation, then a fresh one (n <= 32 < kTcChunk)
+        unsigned long long fresh = 0;
+        if (lane == 0) fresh = atomicAdd(&P.counters[3], (unsigned long long)kTcChunk);
+        fresh = __shfl_sync(0xffffffffu, fresh, 0);
+        if (r >= rec.left) pos = fresh + (unsigned long long)(r - rec.left);
+        const int used = n - rec.left;
+        rec.base = fresh + (unsigned long long)used;
+        rec.left = kTcChunk - used;
+    }
+    if (e.x != 0) {
+        if (pos < (P.band_cap >> 1))
+            reinterpret_cast<int4*>(P.band)[pos] = e;
+        else
+            tc_resolve_here(P, e);
+    }
+}
+
 // DBG: the recording instantiation of the filter dump (a test aid; the join
 // kernels proper carry none of its code).
-template <int KP, bool EMIT, bool DBG>
-__global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams P, TcParams T) {
+template <int KP, bool DBG>
+__global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcParams T) {
     using SH = TcShape<KP>;
-    using SM = TcSmem<KP, EMIT>;
-    constexpr int STAGES = tc_stages<KP, EMIT>();
+    using SM = TcSmem<KP>;
+    constexpr int STAGES = tc_stages<KP>();
     static_assert(STAGES >= 2, "at least two operand stages");
     constexpr int NMAX = SH::NMAX;
     extern __shared__ unsigned char dsm_raw[];
     unsigned char* dsm = reinterpret_cast<unsigned char*>(((uintptr_t)dsm_raw + 1023) & ~(uintptr_t)1023);
     unsigned char* sB = dsm;
-    unsigned char* sA = dsm + SH::B_BYTES;
+    unsigned char* sA = dsm + SH::NB * SH::B_BYTES;
     SM& S = *reinterpret_cast<SM*>(sA + (size_t)STAGES * SH::A_STAGE);
     volatile int* abort = &S.abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -243,17 +322,17 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
             bar_init(&S.a_full[i], 1);
             bar_init(&S.a_empty[i], 1);
         }
-        bar_init(&S.b_full, 1);
-        bar_init(&S.b_empty, 1);
         for (int i = 0; i < 2; ++i) {
+            bar_init(&S.b_full[i], 1);
+            bar_init(&S.b_empty[i], 1);
             bar_init(&S.item_full[i], 1);
-            bar_init(&S.item_empty[i], 1 + SM::EPI);  // the MMA thread and the epilogue warps
+            bar_init(&S.item_empty[i], 2 + SM::EPI);  // the MMA and copy threads and the epilogue warps
             bar_init(&S.acc_full[i], 1);
             bar_init(&S.acc_empty[i], SM::EPI);
         }
         for (int i = 0; i < kMetaDepth; ++i) {
             bar_init(&S.meta_full[i], 1);
-            bar_init(&S.meta_empty[i], SM::EPI);
+            bar_init(&S.meta_empty[i], 1 + SM::EPI);  // the copy thread and the epilogue warps
         }
         bar_init(&S.drain, 1);
         S.abort = 0;
@@ -270,17 +349,14 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
     const uint32_t tmem = S.tmem;
 
     if (warp == 0) {
-        // ------------------------------------------------------------ producer
-        // The whole warp: lane i of a tile resolves the tile's 8-row group i
-        // (a binary search over the item's per-run group prefix), runs of
-        // consecutive groups become one bulk copy per K-slice, issued by the
-        // run's first lane.
-        uint32_t a_i = 0, a_ph = 0, m_i = 0, m_ph = 0, it_i = 0, it_ph = 0, b_ph = 0;
-        uint32_t armed_a[STAGES];  // parity of each stage's last arming + 1 (0: never armed)
-        for (int i = 0; i < STAGES; ++i) armed_a[i] = 0;
-        uint32_t armed_b = 0;
-        int bail = 0;
-        while (!bail) {
+        // ------------------------------------------------------------ tiles
+        // Takes the work items and cuts their candidates into tiles: lane i
+        // of a tile resolves the tile's 8-row group i (a binary search over
+        // the item's per-run group prefix); runs of consecutive groups become
+        // one copy each.  Runs ahead of the copies by the depth of the
+        // metadata ring.
+        uint32_t m_i = 0, m_ph = 0, it_i = 0, it_ph = 0;
+        for (;;) {
             long long it = 0;
             if (lane == 0) it = (long long)atomicAdd(&P.counters[0], 1ull);
             it = __shfl_sync(0xffffffffu, it, 0);
@@ -315,133 +391,141 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
             const int ngroups = carry;
             __syncwarp();
             const int ntiles = (ngroups + kTcG - 1) / kTcG;
-            const int qa = I.q0 & ~7;
-            const int ncol = ((I.q1 - qa) + 15) & ~15;
-            // the ring slot is free once its previous item is done; then its query ids
-            int freed = 1;
-            if (lane == 0) freed = bar_wait(&S.item_empty[it_i], it_ph ^ 1u, abort) ? 1 : 0;
-            freed = __shfl_sync(0xffffffffu, freed, 0);
-            if (freed && it < P.n_items)
-                for (int c = lane; c < ncol; c += 32) {
-                    const int q = qa + c;
-                    S.qperm[it_i][c] = (q >= I.q0 && q < I.q1) ? P.perm[q] : 0;
-                }
-            __syncwarp();
+            // the ring slot is free once its previous item is done
+            if (!bar_wait_warp(&S.item_empty[it_i], it_ph ^ 1u, abort)) break;
             if (lane == 0) {
-                if (!freed) {
-                    bail = 1;
-                } else if (it >= P.n_items) {
-                    S.items[it_i].it = -1;
-                    bar_arrive(&S.item_full[it_i]);
-                    bail = 2;
-                } else {
-                    TcItem& X = S.items[it_i];
-                    X.it = it;
-                    X.q0 = I.q0;
-                    X.q1 = I.q1;
-                    X.qa = qa;
-                    X.ncol = ncol;
-                    X.ntiles = ntiles;
-                    bar_arrive(&S.item_full[it_i]);
-                    // the query tile, one copy per K-slice
-                    if (!bar_wait(&S.b_empty, b_ph ^ 1u, abort)) {
-                        bail = 1;
-                    } else {
-                        const uint32_t gq = (uint32_t)(ncol >> 3);
-                        bar_arrive_tx(&S.b_full, gq * KP * 16u);
-                        armed_b = b_ph + 1;
-                        for (int sl = 0; sl < SH::SLICES; ++sl) {
-                            const int ks = KP - sl * kKS < kKS ? KP - sl * kKS : kKS;
-                            const __nv_bfloat16* src =
-                                T.rows_b + (long long)sl * kKS * T.nrows + (long long)(qa >> 3) * ks * 8;
-                            bulk_g2s(sB + (size_t)NMAX * 2 * kKS * sl, src, gq * (uint32_t)ks * 16u, &S.b_full);
-                        }
-                        b_ph ^= 1u;
-                    }
-                }
+                TcItem& X = S.items[it_i];
+                X.it = it < P.n_items ? it : -1;
+                X.q0 = I.q0;
+                X.q1 = I.q1;
+                X.qa = I.q0 & ~7;
+                X.ncol = ((I.q1 - X.qa) + 15) & ~15;
+                X.ntiles = ntiles;
+                bar_arrive(&S.item_full[it_i]);
             }
-            bail = __shfl_sync(0xffffffffu, bail, 0);
-            if (freed && it < P.n_items && ++it_i == 2) it_i = 0, it_ph ^= 1u;  // (the whole warp)
-            // candidate tiles
-            for (int t = 0; t < ntiles && !bail; ++t) {
-                int w = 1;
-                if (lane == 0) w = bar_wait(&S.meta_empty[m_i], m_ph ^ 1u, abort) ? 1 : 0;
-                if (!__shfl_sync(0xffffffffu, w, 0)) {
-                    bail = 1;
-                    break;
-                }
-                TcMeta& M = S.meta[m_i];
+            if (it >= P.n_items) break;
+            if (++it_i == 2) it_i = 0, it_ph ^= 1u;
+            bool bail = false;
+            for (int t = 0; t < ntiles; ++t) {
                 // this lane's group of the tile
                 const int j = t * kTcG + lane;
-                int32_t g = -1;
-                if (lane < kTcG) {
-                    if (j < ngroups) {
-                        int lo = 0, hi = nr - 1;  // last run whose prefix is <= j
-                        while (lo < hi) {
-                            const int mid = (lo + hi + 1) >> 1;
-                            if (S.rgp[mid] <= j)
-                                lo = mid;
-                            else
-                                hi = mid - 1;
-                        }
-                        g = (S.rlo[lo] >> 3) + (j - S.rgp[lo]);
-                        M.lo[lane] = S.rlo[lo];
-                        M.hi[lane] = S.rhi[lo];
-                        M.fl[lane] = S.rfl[lo];
+                int4 g = make_int4(-8, 0, 0, 0);
+                if (lane < kTcG && j < ngroups) {
+                    int lo = 0, hi = nr - 1;  // last run whose prefix is <= j
+                    while (lo < hi) {
+                        const int mid = (lo + hi + 1) >> 1;
+                        if (S.rgp[mid] <= j)
+                            lo = mid;
+                        else
+                            hi = mid - 1;
                     }
-                    M.g[lane] = g;
+                    g = make_int4((S.rlo[lo] & ~7) + 8 * (j - S.rgp[lo]), S.rlo[lo], S.rhi[lo], S.rfl[lo]);
                 }
                 const int cnt = ngroups - t * kTcG < kTcG ? ngroups - t * kTcG : kTcG;
                 // runs of consecutive groups: their first lanes
-                const int32_t gprev = __shfl_up_sync(0xffffffffu, g, 1);
-                const bool first = lane < cnt && (lane == 0 || g != gprev + 1);
+                const int32_t gprev = __shfl_up_sync(0xffffffffu, g.x, 1);
+                const bool first = lane < cnt && (lane == 0 || g.x != gprev + 8);
                 const uint32_t firsts = __ballot_sync(0xffffffffu, first);
                 const uint32_t later = firsts & ~((2u << lane) - 1u);
                 const int seg_end = later ? __ffs(later) - 1 : cnt;
+                if (!bar_wait_warp(&S.meta_empty[m_i], m_ph ^ 1u, abort)) {
+                    bail = true;
+                    break;
+                }
+                TcMeta& M = S.meta[m_i];
+                if (lane < kTcG) M.g[lane] = g;
+                if (first)
+                    M.seg[__popc(firsts & ((1u << lane) - 1u))] = make_int4(lane, seg_end - lane, g.x >> 3, 0);
+                if (lane == 0) {
+                    M.nseg = __popc(firsts);
+                    M.cnt = cnt;
+                }
                 __syncwarp();
                 if (lane == 0) bar_arrive(&S.meta_full[m_i]);
                 if (++m_i == kMetaDepth) m_i = 0, m_ph ^= 1u;
+            }
+            if (bail) break;
+        }
+    } else if (warp == 2) {
+        // ------------------------------------------------------------ copies
+        // One thread: per item the query tile, per tile and K-slice one bulk
+        // copy for each run of consecutive groups.
+        if (lane == 0) {
+            uint32_t a_i = 0, a_ph = 0, m_i = 0, m_ph = 0, it_i = 0, it_ph = 0, b_i = 0, b_ph = 0;
+            // stages and query tiles armed so far, and the parity of the last arming
+            uint32_t armed_a = 0, par_a = 0, armed_b = 0, par_b = 0;
+            bool bail = false;
+            while (!bail) {
+                if (!bar_wait(&S.item_full[it_i], it_ph, abort)) break;
+                const TcItem X = S.items[it_i];
+                bar_arrive(&S.item_empty[it_i]);
+                if (X.it < 0) break;
+                if (++it_i == 2) it_i = 0, it_ph ^= 1u;
+                // the query tile, one copy per K-slice
+                if (!bar_wait(&S.b_empty[b_i], b_ph ^ 1u, abort)) break;
+                const uint32_t gq = (uint32_t)(X.ncol >> 3);
+                bar_arrive_tx(&S.b_full[b_i], gq * KP * 16u);
+                armed_b |= 1u << b_i;
+                par_b = (par_b & ~(1u << b_i)) | (b_ph << b_i);
                 for (int sl = 0; sl < SH::SLICES; ++sl) {
                     const int ks = KP - sl * kKS < kKS ? KP - sl * kKS : kKS;
-                    if (lane == 0) {
-                        w = bar_wait(&S.a_empty[a_i], a_ph ^ 1u, abort) ? 1 : 0;
-                        if (w) bar_arrive_tx(&S.a_full[a_i], (uint32_t)cnt * ks * 16u);
-                    }
-                    if (!__shfl_sync(0xffffffffu, w, 0)) {
-                        bail = 1;
+                    const __nv_bfloat16* src =
+                        T.rows_b + (long long)sl * kKS * T.nrows + (long long)(X.qa >> 3) * ks * 8;
+                    bulk_g2s(sB + (size_t)b_i * SH::B_BYTES + (size_t)NMAX * 2 * kKS * sl, src, gq * (uint32_t)ks * 16u,
+                             &S.b_full[b_i]);
+                }
+                if (++b_i == SH::NB) b_i = 0, b_ph ^= 1u;
+                for (int t = 0; t < X.ntiles && !bail; ++t) {
+                    if (!bar_wait(&S.meta_full[m_i], m_ph, abort)) {
+                        bail = true;
                         break;
                     }
-                    armed_a[a_i] = a_ph + 1;
-                    if (first) {
-                        unsigned char* dst = sA + (size_t)a_i * SH::A_STAGE + (size_t)lane * ks * 16;
-                        const __nv_bfloat16* src = T.rows_a + (long long)sl * kKS * T.nrows + (long long)g * ks * 8;
-                        bulk_g2s(dst, src, (uint32_t)(seg_end - lane) * ks * 16u, &S.a_full[a_i]);
+                    const TcMeta& M = S.meta[m_i];
+                    const int nseg = M.nseg, cnt = M.cnt;
+                    for (int sl = 0; sl < SH::SLICES; ++sl) {
+                        const int ks = KP - sl * kKS < kKS ? KP - sl * kKS : kKS;
+                        if (!bar_wait(&S.a_empty[a_i], a_ph ^ 1u, abort)) {
+                            bail = true;
+                            break;
+                        }
+                        bar_arrive_tx(&S.a_full[a_i], (uint32_t)cnt * ks * 16u);
+                        armed_a |= 1u << a_i;
+                        par_a = (par_a & ~(1u << a_i)) | (a_ph << a_i);
+                        unsigned char* dst = sA + (size_t)a_i * SH::A_STAGE;
+                        const __nv_bfloat16* src = T.rows_a + (long long)sl * kKS * T.nrows;
+                        for (int k = 0; k < nseg; ++k) {
+                            const int4 e = M.seg[k];
+                            bulk_g2s(dst + (size_t)e.x * ks * 16, src + (long long)e.z * ks * 8,
+                                     (uint32_t)e.y * ks * 16u, &S.a_full[a_i]);
+                        }
+                        if (++a_i == STAGES) a_i = 0, a_ph ^= 1u;
                     }
-                    if (++a_i == STAGES) a_i = 0, a_ph ^= 1u;
+                    bar_arrive(&S.meta_empty[m_i]);
+                    if (++m_i == kMetaDepth) m_i = 0, m_ph ^= 1u;
                 }
             }
-        }
-        if (*abort && lane == 0) {
-            // drain the copies this CTA armed (bounded), so none lands after exit
-            for (int i = 0; i < STAGES; ++i)
-                if (armed_a[i])
-                    for (long long k = 0; k < kTcSpin && !bar_test(&S.a_full[i], armed_a[i] - 1); ++k) {
-                    }
-            if (armed_b)
-                for (long long k = 0; k < kTcSpin && !bar_test(&S.b_full, armed_b - 1); ++k) {
-                }
+            if (*abort) {
+                // drain the copies this CTA armed (bounded), so none lands after exit
+                for (int i = 0; i < STAGES; ++i)
+                    if (armed_a >> i & 1u)
+                        for (long long k = 0; k < kTcSpin && !bar_test(&S.a_full[i], par_a >> i & 1u); ++k) {
+                        }
+                for (int i = 0; i < SH::NB; ++i)
+                    if (armed_b >> i & 1u)
+                        for (long long k = 0; k < kTcSpin && !bar_test(&S.b_full[i], par_b >> i & 1u); ++k) {
+                        }
+            }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            uint32_t a_i = 0, a_ph = 0, it_i = 0, it_ph = 0, b_ph = 0, acc = 0, acc_ph = 0;
+            uint32_t a_i = 0, a_ph = 0, it_i = 0, it_ph = 0, b_i = 0, b_ph = 0, acc = 0, acc_ph = 0;
             bool issued = false;
             for (;;) {
                 if (!bar_wait(&S.item_full[it_i], it_ph, abort)) break;
                 const TcItem X = S.items[it_i];
                 if (X.it < 0) break;
-                if (!bar_wait(&S.b_full, b_ph, abort)) break;
-                b_ph ^= 1u;
+                if (!bar_wait(&S.b_full[b_i], b_ph, abort)) break;
                 const uint32_t idesc = umma_idesc(kTcM, X.ncol, T.ab_bf16);
                 bool fail = false;
                 for (int t = 0; t < X.ntiles && !fail; ++t) {
@@ -459,7 +543,7 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
                         }
                         asm volatile("tcgen05.fence::after_thread_sync;");
                         const uint32_t a0 = smem_u32(sA + (size_t)a_i * SH::A_STAGE);
-                        const uint32_t b0 = smem_u32(sB + (size_t)NMAX * 2 * kKS * sl);
+                        const uint32_t b0 = smem_u32(sB + (size_t)b_i * SH::B_BYTES + (size_t)NMAX * 2 * kKS * sl);
                         for (int kk = 0; kk < ks / 16; ++kk) {
                             const uint64_t ad = umma_desc(a0 + kk * 256, 128, (uint32_t)ks * 16u);
                             const uint64_t bd = umma_desc(b0 + kk * 256, 128, (uint32_t)ks * 16u);
@@ -478,7 +562,8 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
                     if (++acc == 2) acc = 0, acc_ph ^= 1u;
                 }
                 if (fail) break;
-                umma_commit(&S.b_empty);  // the query tile is free once this item's MMAs are done
+                umma_commit(&S.b_empty[b_i]);  // the query tile is free once this item's MMAs are done
+                if (++b_i == SH::NB) b_i = 0, b_ph ^= 1u;
                 bar_arrive(&S.item_empty[it_i]);
                 if (++it_i == 2) it_i = 0, it_ph ^= 1u;
             }
@@ -491,38 +576,33 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
         }
     } else {
         // ------------------------------------------------------------ epilogue
-        const int ew = warp - 2;       // stage slot
+        const int ew = warp - 3;
         const int quarter = warp & 3;  // TMEM lanes 32 quarter .. + 31
         const int part = ew >> 2;      // 32-column chunks part, part + EPI / 4, ...
         const int row = quarter * 32 + lane;
         const float* __restrict__ TO = static_cast<const float*>(P.thr_out);
         const float* __restrict__ TI = static_cast<const float*>(P.thr_in);
-        WarpStage st{S.stage[ew], EMIT ? S.sdist[ew] : nullptr, 0, 0};
-        BandQ bq{0, 0};
-        unsigned long long rechecked = 0;
+        TcRecords rec{0, 0};
         uint32_t it_i = 0, it_ph = 0, m_i = 0, m_ph = 0, acc = 0, acc_ph = 0;
         for (;;) {
-            if (!bar_wait(&S.item_full[it_i], it_ph, abort)) break;
+            if (!bar_wait_warp(&S.item_full[it_i], it_ph, abort)) break;
             const TcItem X = S.items[it_i];
             if (X.it < 0) break;
-            const ItemRoute R = item_route(st, P, X.it, lane);
             bool fail = false;
             // this thread's candidate row, read one tile ahead so its
             // threshold loads overlap the previous tile
-            int32_t p = 0, pid = 0;
+            int32_t p = 0;
             bool valid = false;
             int fl = 0;
             float to = INFINITY, ti = INFINITY;
-            const int32_t* qperm = S.qperm[it_i];
             auto read_meta = [&]() -> bool {
-                if (!bar_wait(&S.meta_full[m_i], m_ph, abort)) return false;
+                if (!bar_wait_warp(&S.meta_full[m_i], m_ph, abort)) return false;
                 const TcMeta& M = S.meta[m_i];
-                const int gi = row >> 3;
-                const int32_t g = M.g[gi];
-                p = g * 8 + (row & 7);
-                if (g >= 0 && !SJ_BOUND(P, p < P.n_points + kTcPadRows, 31)) p = 0;
-                valid = g >= 0 && p >= M.lo[gi] && p < M.hi[gi];
-                fl = M.fl[gi];
+                const int4 g = M.g[row >> 3];
+                p = g.x + (row & 7);
+                if (g.x >= 0 && !SJ_BOUND(P, p < P.n_points + kTcPadRows, 31)) p = 0;
+                valid = g.x >= 0 && p >= g.y && p < g.z;
+                fl = g.w;
                 __syncwarp();
                 if (lane == 0) bar_arrive(&S.meta_empty[m_i]);
                 if (++m_i == kMetaDepth) m_i = 0, m_ph ^= 1u;
@@ -533,115 +613,112 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
                 const int32_t pl = valid ? p : 0;
                 to = TO[pl];
                 ti = TI[pl];
-                pid = P.perm[pl];
                 return true;
             };
             if (X.ntiles > 0 && !read_meta()) fail = true;
             const int cq0 = X.q0 - X.qa, cq1 = X.q1 - X.qa;  // the item's query columns
             for (int t = 0; t < X.ntiles && !fail; ++t) {
-                const int32_t cp = p, cpid = pid;
+                const int32_t cp = p;
                 const bool cvalid = valid;
                 const int cfl = fl;
-                const float cto = to, cti = ti;
+                const float cto = to;
+                // negated thresholds, never -0: the sign of a round-to-nearest
+                // sum a + nto is that of the exact a - cto
+                const float nto = __fsub_rn(0.f, to), nti = __fsub_rn(0.f, ti);
                 // this row's valid query columns: the item's, and in a self-cell
                 // triangle those at or below the candidate (one unsigned compare)
                 const int col_lo = cq0;
                 const int col_hi = cfl == 2 ? min(cq1 - 1, cp - X.qa) : cq1 - 1;
                 const bool has_cols = col_hi >= col_lo;
                 const uint32_t col_span = has_cols ? (uint32_t)(col_hi - col_lo) : 0u;
-                if (!bar_wait(&S.acc_full[acc], acc_ph, abort)) {
+                if (!bar_wait_warp(&S.acc_full[acc], acc_ph, abort)) {
                     fail = true;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;");
-                if (t + 1 < X.ntiles && !read_meta()) {
-                    fail = true;
-                    break;
-                }
-                // this lane's maybe-in columns of a 32-column chunk (column | certain << 8),
-                // emitted afterwards a warp-wide round at a time
-                uint16_t(*hits)[32] = S.hits[ew];
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + acc * NMAX;
-                for (int c0 = 32 * part; c0 < X.ncol; c0 += 32 * (SM::EPI / 4)) {
-                    // only the N accumulated columns are read (a 16-column tail
-                    // leaves the upper half at -inf)
-                    uint32_t v[32];
-                    if (X.ncol - c0 == 16) {
-                        tmem_ld16(taddr + (uint32_t)c0, v);
+                constexpr int CSTEP = 32 * (SM::EPI / 4), UN = tc_chunks(KP);
+                // UN chunks at a time, their loads and the next tile's metadata
+                // in flight together; the accumulator is released as soon as
+                // this warp's last columns are in registers, before any of
+                // them is looked at
+                for (int c0 = 32 * part; c0 < X.ncol || c0 == 32 * part; c0 += UN * CSTEP) {
+                    // (whole chunks, no branches around the loads: columns past
+                    // the accumulated ones hold an earlier tile's and are left
+                    // out below)
+                    bool live[UN];
+                    uint32_t v[UN][32];
 #pragma unroll
-                        for (int k = 16; k < 32; ++k) v[k] = 0xFF800000u;
-                    } else {
-                        tmem_ld32(taddr + (uint32_t)c0, v);
+                    for (int u = 0; u < UN; ++u) {
+                        live[u] = c0 + u * CSTEP < X.ncol;
+                        tmem_ld32(taddr + (uint32_t)(live[u] ? c0 + u * CSTEP : 32 * part), v[u]);
                     }
+                    if (c0 == 32 * part && t + 1 < X.ntiles && !read_meta()) fail = true;
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (X.ncol - c0 <= UN * CSTEP) {  // (this warp's last chunks)
+                        asm volatile("tcgen05.fence::before_thread_sync;");
+                        __syncwarp();
+                        if (lane == 0) bar_arrive(&S.acc_empty[acc]);
+                    }
                     if (DBG && cvalid && has_cols) {  // the filter dump (test aid)
                         // (constant indices: v stays in registers)
 #pragma unroll
-                        for (int k = 0; k < 32; ++k) {
-                            const int col = c0 + k;
-                            if (col < X.ncol && (uint32_t)(col - col_lo) <= col_span)
-                                dbg_record(P, X.qa + col, cp, __uint_as_float(v[k]));
-                        }
-                    }
-                    // maxima of 8-column groups, then of all 32 (three-input max)
-                    float m8[4];
+                        for (int u = 0; u < UN; ++u)
 #pragma unroll
-                    for (int g8 = 0; g8 < 4; ++g8) {
-                        const float* f = reinterpret_cast<const float*>(v + 8 * g8);
-                        m8[g8] = max3f(max3f(f[0], f[1], f[2]), max3f(f[3], f[4], f[5]), fmaxf(f[6], f[7]));
-                    }
-                    const float mall = max3f(m8[0], m8[1], fmaxf(m8[2], m8[3]));
-                    if (!__any_sync(0xffffffffu, cvalid && mall >= cto)) continue;
-                    int hn = 0;
-#pragma unroll
-                    for (int g8 = 0; g8 < 4; ++g8) {
-                        const bool h = cvalid && m8[g8] >= cto;
-                        if (!__any_sync(0xffffffffu, h)) continue;
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const int col = c0 + 8 * g8 + k;
-                            const float a = __uint_as_float(v[8 * g8 + k]);
-                            const bool ok = h && has_cols && a >= cto && (uint32_t)(col - col_lo) <= col_span;
-                            if (ok) hits[hn++][lane] = (uint16_t)((uint32_t)col | (a >= cti ? 256u : 0u));
-                        }
-                    }
-                    for (int i = 0; __any_sync(0xffffffffu, i < hn); ++i) {
-                        int nout = 0;
-                        int32_t qid = 0, cid = 0, qs = 0;
-                        double dist = 0.0;
-                        bool band = false, mir = false;
-                        if (i < hn) {
-                            const uint32_t e = hits[i][lane];
-                            qs = X.qa + (int)(e & 255u);
-                            mir = cfl == 1 || (cfl == 2 && cp != qs);
-                            if ((e >> 8) && !EMIT) {
-                                nout = mir ? 2 : 1;
-                                qid = (int32_t)(qperm[qs - X.qa] - R.off);
-                                cid = (int32_t)(cpid - R.off);
-                            } else {
-                                band = true;
+                            for (int k = 0; k < 32; ++k) {
+                                const int col = c0 + u * CSTEP + k;
+                                if (col < X.ncol && (uint32_t)(col - col_lo) <= col_span)
+                                    dbg_record(P, X.qa + col, cp, __uint_as_float(v[u][k]));
                             }
-                        }
-                        const bool queued = band_push_q(bq, P, lane, band, qs, cp, mir);
-                        if (band && !queued) {  // queue full: decide here
-                            const double s2 = direct_sq(P.xs + (int64_t)qs * P.dp, P.xs + (int64_t)cp * P.dp, P.d);
-                            ++rechecked;
-                            if (s2 <= R.e2) {
-                                nout = mir ? 2 : 1;
-                                qid = (int32_t)(qperm[qs - X.qa] - R.off);
-                                cid = (int32_t)(cpid - R.off);
-                                if (EMIT) dist = sqrt(s2);
+                    }
+                    // maxima of 8-column groups, then of all 32 (three-input
+                    // max), of all chunks before one is acted on
+                    float m8[UN][4];
+                    bool any[UN];
+#pragma unroll
+                    for (int u = 0; u < UN; ++u) {
+                        const float* f = reinterpret_cast<const float*>(v[u]);
+#pragma unroll
+                        for (int g8 = 0; g8 < 4; ++g8)
+                            m8[u][g8] = max3f(max3f(f[8 * g8], f[8 * g8 + 1], f[8 * g8 + 2]),
+                                              max3f(f[8 * g8 + 3], f[8 * g8 + 4], f[8 * g8 + 5]),
+                                              fmaxf(f[8 * g8 + 6], f[8 * g8 + 7]));
+                        if (X.ncol - (c0 + u * CSTEP) < 32) m8[u][2] = m8[u][3] = -INFINITY;  // (a 16-column tail)
+                    }
+#pragma unroll
+                    for (int u = 0; u < UN; ++u)
+                        any[u] = __any_sync(0xffffffffu, live[u] && cvalid &&
+                                                          max3f(m8[u][0], m8[u][1], fmaxf(m8[u][2], m8[u][3])) >= cto);
+#pragma unroll
+                    for (int u = 0; u < UN; ++u) {
+                        const int cu = c0 + u * CSTEP;
+                        if (!any[u]) continue;
+                        const float* f = reinterpret_cast<const float*>(v[u]);
+                        // bit k: column cu + k is maybe in / certainly in
+                        uint32_t mo = 0u, mi = 0u;
+#pragma unroll
+                        for (int g8 = 0; g8 < 4; ++g8) {
+                            if (!__any_sync(0xffffffffu, cvalid && m8[u][g8] >= cto)) continue;
+                            // sign of a - threshold (see nto): a miss
+                            uint32_t no = 0u, ni = 0u;
+#pragma unroll
+                            for (int k = 6; k >= 0; k -= 2) {
+                                const float2 a = make_float2(f[8 * g8 + k], f[8 * g8 + k + 1]);
+                                const float2 o = __fadd2_rn(a, make_float2(nto, nto));
+                                const float2 n = __fadd2_rn(a, make_float2(nti, nti));
+                                no = push_sign(push_sign(no, o.y), o.x);
+                                ni = push_sign(push_sign(ni, n.y), n.x);
                             }
+                            mo |= (~no & 0xFFu) << (8 * g8);
+                            mi |= (~ni & 0xFFu) << (8 * g8);
                         }
-                        if (EMIT)
-                            stage_emit(st, P, lane, nout, qid, cid, dist);
-                        else
-                            stage_emit_pairs(st, P, lane, nout, qid, cid);
+                        // this row's columns (the item's, the triangle's)
+                        const int lo = max(col_lo - cu, 0), hi = min(col_hi - cu, 31);
+                        mo &= cvalid && lo <= hi ? (0xFFFFFFFFu << lo) & (0xFFFFFFFFu >> (31 - hi)) : 0u;
+                        tc_record(rec, P, lane, make_int4((int)mo, (int)mi, X.qa + cu,
+                                                          (int)((uint32_t)cp | (cfl ? kMirrorBit : 0u))));
                     }
                 }
-                asm volatile("tcgen05.fence::before_thread_sync;");
-                __syncwarp();
-                if (lane == 0) bar_arrive(&S.acc_empty[acc]);
                 if (++acc == 2) acc = 0, acc_ph ^= 1u;
             }
             if (fail) break;
@@ -649,10 +726,10 @@ __global__ void __launch_bounds__(tc_threads(KP, EMIT), 1) k_join_tc(JoinParams 
             if (lane == 0) bar_arrive(&S.item_empty[it_i]);
             if (++it_i == 2) it_i = 0, it_ph ^= 1u;
         }
-        band_q_close(bq, P, lane);
-        stage_flush(st, P, lane);
-        for (int o = 16; o > 0; o >>= 1) rechecked += __shfl_down_sync(0xffffffffu, rechecked, o);
-        if (lane == 0 && rechecked) atomicAdd(&P.counters[2], rechecked);
+        // the warp's unfilled records are closed (no columns)
+        for (int i = lane; i < rec.left; i += 32)
+            if (rec.base + (unsigned long long)i < (P.band_cap >> 1))
+                reinterpret_cast<int4*>(P.band)[rec.base + (unsigned long long)i] = make_int4(0, 0, 0, 0);
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -702,17 +779,17 @@ int selftest_bounded_wait(cudaStream_t s) {
     return SJ_ERR_CUDA;
 }
 
-template <int KP, bool EMIT, bool DBG = false>
+template <int KP, bool DBG>
 static int launch_kp(Index* ix, const JoinParams& p, const TcParams& t) {
-    auto kern = k_join_tc<KP, EMIT, DBG>;
-    const size_t smem = tc_smem_bytes<KP, EMIT>();
+    auto kern = k_join_tc<KP, DBG>;
+    const size_t smem = tc_smem_bytes<KP>();
     if (smem > kSmemMax) {
         set_error("tensor-core tile does not fit in shared memory (K = %d)", KP);
         return SJ_ERR_UNSUPPORTED;
     }
     SJ_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    constexpr int threads = tc_threads(KP, EMIT);
+    constexpr int threads = tc_threads(KP);
     SJ_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     if (per_sm < 1) {
         set_error("tensor-core tile does not fit on an SM (K = %d)", KP);
@@ -729,8 +806,7 @@ static int launch_kp(Index* ix, const JoinParams& p, const TcParams& t) {
 
 template <int KP>
 static int launch_k(Index* ix, const JoinParams& p, const TcParams& t) {
-    if (p.dbg) return launch_kp<KP, false, true>(ix, p, t);  // the filter dump (no distances)
-    return p.emit_dist ? launch_kp<KP, true>(ix, p, t) : launch_kp<KP, false>(ix, p, t);
+    return p.dbg ? launch_kp<KP, true>(ix, p, t) : launch_kp<KP, false>(ix, p, t);  // (dbg: the filter dump)
 }
 
 int launch_join_tc(Index* ix, const JoinOut& out, int emit_dist) {

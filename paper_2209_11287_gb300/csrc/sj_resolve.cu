@@ -1,0 +1,183 @@
+// What the tensor-core filter leaves open: its records (one candidate against
+// up to 32 query positions, see sj_join_tc.cu) become result pairs.
+//
+// The filter's tile kernel only finds the maybe-in pairs and appends a record
+// where there are any; deciding and emitting them there kept each epilogue warp
+// in long serial code while its accumulator waited (16-D mixture, 500,000
+// points: 2.2 of 5.2 ms).  Here they are spread over the whole chip: a warp
+// expands 32 records into a list and deals with 32 pairs at a time.
+//
+// A pair that the filter's bound does not certify is first evaluated in
+// binary32 by the direct form on the kernel coordinates, sum of (y_q - y_c)^2.
+// That sum's error is relative to the distance, not to the norms of the points
+// as in the expanded form, so nearly every pair is certified out or in by it
+// (refine_out, refine_in; pack_coefficients), at FP32 rate; binary64, which
+// runs at 1/64 of that, decides the rest and gives the distances.  Measured
+// against rechecking every such pair in binary64 (k_recheck, with the emission
+// of the certain pairs still in the tile kernel): 500,000 x 16-D mixture (7.3 M
+// uncertain of 28 M pairs) 703 / 380 us, 200,000 x 64-D 586 / 210 us.  Bound by
+// the gathers of rows and ids and the emission.
+#include "sj_join_common.cuh"
+
+namespace sj {
+
+namespace {
+
+constexpr int kResolveWarps = 4;
+
+// Squared distance of two kernel-coordinate rows, binary32.
+template <int DP>
+__device__ __forceinline__ float refine_sq(const float* __restrict__ a, const float* __restrict__ b) {
+    float s = 0.f;
+    if constexpr (DP < 4) {
+#pragma unroll
+        for (int k = 0; k < DP; ++k) {
+            const float t = a[k] - b[k];
+            s = __fmaf_rn(t, t, s);
+        }
+    } else {
+#pragma unroll 4
+        for (int k = 0; k < DP / 4; ++k) {
+            const float4 u = reinterpret_cast<const float4*>(a)[k], v = reinterpret_cast<const float4*>(b)[k];
+            const float t0 = u.x - v.x, t1 = u.y - v.y, t2 = u.z - v.z, t3 = u.w - v.w;
+            s = __fmaf_rn(t0, t0, s);
+            s = __fmaf_rn(t1, t1, s);
+            s = __fmaf_rn(t2, t2, s);
+            s = __fmaf_rn(t3, t3, s);
+        }
+    }
+    return s;
+}
+
+template <int DP, bool EMIT>
+__global__ void __launch_bounds__(32 * kResolveWarps) k_resolve(JoinParams P) {
+    __shared__ int2 s_stage[kResolveWarps][kStage];
+    __shared__ double s_sdist[kResolveWarps][EMIT ? kStage : 1];
+    // pairs waiting: (query position | certain << 31, candidate position | mirrored << 31)
+    __shared__ int2 s_list[kResolveWarps][64];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const float* __restrict__ Y = static_cast<const float*>(P.y);
+    WarpStage st{s_stage[wid], EMIT ? s_sdist[wid] : nullptr, 0, 0};
+    int2* list = s_list[wid];
+    int waiting = 0;
+    unsigned long long decided = 0;
+
+    // 32 pairs, one a lane
+    auto deal = [&](bool live, int2 e) {
+        const int32_t qs = (int32_t)((uint32_t)e.x & ~kMirrorBit), cs = (int32_t)((uint32_t)e.y & ~kMirrorBit);
+        live = live && SJ_BOUND(P, qs < P.n_points && cs < P.n_points, 41);
+        const bool certain = !EMIT && e.x < 0;
+        int nout = 0, gid = 0;
+        int32_t qid = 0, cid = 0, off = 0;
+        double dist = 0.0;
+        if (live) {
+            float r_out = P.refine_out, r_in = P.refine_in;
+            double e2 = P.e2;
+            if (P.batch) {
+                const int li = P.batch->inst_of_sorted[qs];
+                const float2 r = P.batch->inst_refine[li];
+                r_out = r.x;
+                r_in = r.y;
+                e2 = P.batch->inst_e2[li];
+                gid = P.batch->inst_gid[li];
+                off = (int32_t)P.batch->inst_off[li];
+            }
+            bool in = certain;
+            if (!certain) {
+                ++decided;
+                const float s32 = refine_sq<DP>(Y + (int64_t)qs * DP, Y + (int64_t)cs * DP);
+                in = s32 < r_in;
+                if (EMIT ? !(s32 > r_out) : !in && !(s32 > r_out)) {
+                    const double s = direct_sq(P.xs + (int64_t)qs * DP, P.xs + (int64_t)cs * DP, P.d);
+                    in = s <= e2;
+                    if (EMIT && in) dist = sqrt(s);
+                }
+            }
+            if (in) {
+                nout = e.y < 0 && cs != qs ? 2 : 1;
+                qid = P.perm[qs] - off;
+                cid = P.perm[cs] - off;
+            }
+        }
+        if (P.batch) {
+            // the pairs of a warp nearly always belong to one instance: they
+            // share its stage; otherwise each lane writes its own
+            const unsigned some = __ballot_sync(0xffffffffu, nout > 0);
+            if (some == 0u) return;
+            const int g0 = __shfl_sync(0xffffffffu, gid, __ffs(some) - 1);
+            if (!__all_sync(0xffffffffu, nout == 0 || gid == g0)) {
+                if (nout > 0) batch_emit_one(P, gid, nout, qid, cid, dist);
+                __syncwarp();
+                return;
+            }
+            if (st.cnt > 0 && st.gid != g0) stage_flush(st, P, lane);
+            st.gid = g0;
+        }
+        if (EMIT)
+            stage_emit(st, P, lane, nout, qid, cid, dist);
+        else
+            stage_emit_pairs(st, P, lane, nout, qid, cid);
+    };
+
+    const int4* __restrict__ records = reinterpret_cast<const int4*>(P.band);
+    const unsigned long long taken = P.counters[3], room = P.band_cap >> 1;
+    const unsigned long long count = taken < room ? taken : room;
+    const unsigned long long step = (unsigned long long)gridDim.x * kResolveWarps * 32;
+    for (unsigned long long b = ((unsigned long long)blockIdx.x * kResolveWarps + wid) * 32; b < count; b += step) {
+        const int4 e = b + lane < count ? records[b + lane] : make_int4(0, 0, 0, 0);
+        uint32_t m = (uint32_t)e.x;
+        for (;;) {  // a column of every record at a time into the list
+            const unsigned w = __ballot_sync(0xffffffffu, m != 0u);
+            if (w == 0u) break;
+            if (m) {
+                const int k = __ffs(m) - 1;
+                m &= m - 1u;
+                list[waiting + __popc(w & ((1u << lane) - 1u))] =
+                    make_int2((int)((uint32_t)(e.z + k) | ((uint32_t)e.y >> k & 1u) << 31), e.w);
+            }
+            waiting += __popc(w);
+            if (waiting >= 32) {
+                waiting -= 32;
+                __syncwarp();
+                deal(true, list[waiting + lane]);
+                __syncwarp();
+            }
+        }
+    }
+    __syncwarp();
+    deal(lane < waiting, list[lane < waiting ? lane : 0]);
+    stage_flush(st, P, lane);
+    for (int o = 16; o > 0; o >>= 1) decided += __shfl_down_sync(0xffffffffu, decided, o);
+    if (lane == 0 && decided) atomicAdd(&P.counters[2], decided);
+}
+
+template <int DP>
+int launch_resolve_dp(Index* ix, const JoinParams& p) {
+    const unsigned blocks = (unsigned)device_sm_count(ix->device) * 8;
+    if (p.emit_dist)
+        k_resolve<DP, true><<<blocks, 32 * kResolveWarps, 0, ix->stream>>>(p);
+    else
+        k_resolve<DP, false><<<blocks, 32 * kResolveWarps, 0, ix->stream>>>(p);
+    note_launch();
+    SJ_CK(cudaGetLastError());
+    return SJ_OK;
+}
+
+}  // namespace
+
+int launch_resolve(Index* ix, const JoinOut& out, int emit_dist) {
+    const JoinParams p = make_join_params(ix, out, emit_dist);
+    switch (ix->dp) {
+        case 2: return launch_resolve_dp<2>(ix, p);
+        case 4: return launch_resolve_dp<4>(ix, p);
+        case 8: return launch_resolve_dp<8>(ix, p);
+        case 16: return launch_resolve_dp<16>(ix, p);
+        case 32: return launch_resolve_dp<32>(ix, p);
+        case 64: return launch_resolve_dp<64>(ix, p);
+        default:
+            set_error("no record resolution for padded dimension %d", ix->dp);
+            return SJ_ERR_UNSUPPORTED;
+    }
+}
+
+}  // namespace sj
