@@ -158,6 +158,17 @@ bool is_device_pointer(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Device memory (not managed) of the calling thread's current device.
+static bool on_current_device(const void* p) {
+    cudaPointerAttributes a{};
+    int dev = 0;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 int side_stream(int device, cudaStream_t* out) {
     static std::mutex mu;
     static cudaStream_t streams[64];
@@ -227,6 +238,56 @@ int round_dim(int d) {
     int p = 2;
     while (p < d) p <<= 1;
     return p;
+}
+
+// Gathers result pages (of 2^log2 8-byte elements each) into one array.
+struct PageList {
+    static constexpr int kMax = 448;  // 3.5 KB of kernel parameters
+    const double* page[kMax];
+};
+__global__ void __launch_bounds__(256) k_gather_pages(PageList pages, int log2, long long count, double* out) {
+    const long long mask = (1ll << log2) - 1;
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < count; i += gridDim.x * 256ll)
+        out[i] = pages.page[i >> log2][i & mask];
+}
+
+// Copies the first `held` elements (8 bytes: a pair, a distance) of a result's
+// pages to `out`, host or device.  Pages that follow one another in the pool
+// are one copy (all of a single join's).  The pages of a batched instance lie
+// scattered between those of others: into device memory they are gathered by
+// one kernel per PageList::kMax pages instead of a copy each (96 instances,
+// 589 pages of 512 KB, a call per instance: 4.3 / 1.6 ms).
+template <typename T>
+static int copy_pages(const T* const* pages, int n_pages, int64_t page_pairs, int64_t held, T* out, cudaStream_t s) {
+    static_assert(sizeof(T) == 8, "elements of 8 bytes");
+    std::vector<int> cut;  // first page of each copy
+    for (int p = 0; (int64_t)p * page_pairs < held; ++p)
+        if (p == 0 || pages[p] != pages[p - 1] + page_pairs) cut.push_back(p);
+    const int used = (int)((held + page_pairs - 1) / page_pairs);
+    if (cut.size() > 2 && (page_pairs & (page_pairs - 1)) == 0 && (reinterpret_cast<uintptr_t>(out) & 7u) == 0 &&
+        on_current_device(out) && on_current_device(pages[0])) {
+        int log2 = 0, dev = 0;
+        while ((int64_t(1) << log2) < page_pairs) ++log2;
+        SJ_CK(cudaGetDevice(&dev));
+        for (int p0 = 0; p0 < used; p0 += PageList::kMax) {
+            PageList list;
+            const int np = std::min(used - p0, PageList::kMax);
+            for (int p = 0; p < np; ++p) list.page[p] = reinterpret_cast<const double*>(pages[p0 + p]);
+            const long long cnt = std::min<int64_t>(held - (int64_t)p0 * page_pairs, (int64_t)np * page_pairs);
+            const long long blocks = std::min<long long>((cnt + 1023) / 1024, (long long)device_sm_count(dev) * 8);
+            k_gather_pages<<<(unsigned)blocks, 256, 0, s>>>(list, log2, cnt,
+                                                           reinterpret_cast<double*>(out + (int64_t)p0 * page_pairs));
+            note_launch();
+            SJ_CK(cudaGetLastError());
+        }
+        return SJ_OK;
+    }
+    for (size_t c = 0; c < cut.size(); ++c) {
+        const int64_t from = (int64_t)cut[c] * page_pairs;
+        const int64_t to = c + 1 < cut.size() ? (int64_t)cut[c + 1] * page_pairs : held;
+        SJ_CK(cudaMemcpyAsync(out + from, pages[cut[c]], (size_t)(to - from) * sizeof(T), cudaMemcpyDefault, s));
+    }
+    return SJ_OK;
 }
 
 }  // namespace sj
@@ -893,18 +954,12 @@ int sj_result_copy(const sj_result* r, int32_t* pairs_out, double* dist_out) {
         set_error("result has no pages");
         return SJ_ERR_ARG;
     }
-    int64_t left = std::min<int64_t>(r->count, (int64_t)r->n_pages * r->page_pairs);
-    for (int p = 0; p < r->n_pages && left > 0; ++p) {
-        const int64_t cnt = std::min<int64_t>(left, r->page_pairs);
-        const int64_t off = (int64_t)p * r->page_pairs;
-        if (pairs_out)
-            SJ_CK(cudaMemcpyAsync(pairs_out + 2 * off, r->pair_pages[p], (size_t)cnt * 2 * sizeof(int32_t),
-                                  cudaMemcpyDefault, ri->stream));
-        if (dist_out && r->has_distances && r->dist_pages)
-            SJ_CK(cudaMemcpyAsync(dist_out + off, r->dist_pages[p], (size_t)cnt * sizeof(double), cudaMemcpyDefault,
-                                  ri->stream));
-        left -= cnt;
-    }
+    const int64_t held = std::min<int64_t>(r->count, (int64_t)r->n_pages * r->page_pairs);
+    if (pairs_out)
+        SJ_TRY(copy_pages(reinterpret_cast<const int2* const*>(r->pair_pages), r->n_pages, r->page_pairs, held,
+                          reinterpret_cast<int2*>(pairs_out), ri->stream));
+    if (dist_out && r->has_distances && r->dist_pages)
+        SJ_TRY(copy_pages(r->dist_pages, r->n_pages, r->page_pairs, held, dist_out, ri->stream));
     SJ_CK(cudaStreamSynchronize(ri->stream));
     return SJ_OK;
 }
