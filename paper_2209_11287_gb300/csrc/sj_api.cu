@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(256) k_gather_pages(PageList pages, int log2, 
 // are one copy (all of a single join's).  The pages of a batched instance lie
 // scattered between those of others: into device memory they are gathered by
 // one kernel per PageList::kMax pages instead of a copy each (96 instances,
-// 589 pages of 512 KB, a call per instance: 4.3 / 1.6 ms).
+// 589 pages of 512 KB, a call per instance: 4.3 / 2.4 ms).
 template <typename T>
 static int copy_pages(const T* const* pages, int n_pages, int64_t page_pairs, int64_t held, T* out, cudaStream_t s) {
     static_assert(sizeof(T) == 8, "elements of 8 bytes");

@@ -1077,6 +1077,201 @@ __global__ void k_denum(DenseEnum e, const unsigned long long* __restrict__ off6
     }
 }
 
+// k_denum for grids of m >= 4 indexed dims (27, 81 or 243 runs a cell), a warp a
+// cell: the lanes take the offset vectors, 32 at a time, and keep their order
+// by ballots.  One thread a cell walked all offsets alone, two dependent loads
+// each, in warps of which most lanes had an empty cell: 500,000 x 16-D mixture
+// (6,572 of 1.77 M keys occupied, 243 offsets, count and fill pass) 580 us,
+// now 142; 100,000 of it 469 / 74; 19 cells of 64-D 120 / 29; with every key
+// occupied and 27 offsets (2 M and 1 M x 4-D) as before, 50 / 51 and 209 / 198.
+// Lanes first load the keys of 32 cells and decode their coordinates; the
+// occupied ones are then done one after another.  A block runs over many keys,
+// so the totals take five atomics a block (one address each for the whole
+// grid: 200,000 of them cost more than the runs where every key is occupied).
+// The offsets are the same as k_denum's, in the same order.  (m <= 3: at most 9
+// offsets, a third of a warp: a thread a cell.)
+constexpr int kDenumWarps = 4;
+template <int MODE>
+__global__ void __launch_bounds__(32 * kDenumWarps) k_denum_warp(DenseEnum e, const unsigned long long* __restrict__ off64,
+                                                                 uint32_t* run_cnt, const uint32_t* __restrict__ run_off,
+                                                                 Run* runs, Item* items, DenseTotals* tot,
+                                                                 uint32_t slots) {
+    constexpr bool FILL = MODE >= 1;
+    constexpr bool COUNT = MODE != 1;
+    __shared__ int32_t s_delta[243];  // per offset vector: the key difference,
+    __shared__ uint16_t s_off[243];   // the offsets + 1 (2 bits a dim) | sign << 12 (0: zero vector, 1: positive, 2: negative)
+    __shared__ unsigned long long s_tot[5];
+    const int lane = threadIdx.x & 31;
+    const int mm = e.m - 1;
+    int nvec = 1;
+    for (int k = 0; k < mm; ++k) nvec *= 3;
+    for (int vi = threadIdx.x; vi < nvec; vi += blockDim.x) {
+        int rem = vi, sign = 0, delta = 0;
+        uint32_t packed = 0;
+        for (int k = 0; k < mm; ++k) {
+            const int o = rem % 3 - 1;
+            rem /= 3;
+            if (sign == 0) sign = o;
+            delta += o * (int)e.stride[k];  // (the key space is below 2^31)
+            packed |= (uint32_t)(o + 1) << (2 * k);
+        }
+        s_delta[vi] = delta;
+        s_off[vi] = (uint16_t)(packed | (uint32_t)(sign > 0 ? 1 : sign < 0 ? 2 : 0) << 12);
+    }
+    if (threadIdx.x < 5) s_tot[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned long long my_eval = 0, my_sq = 0, my_skip = 0, my_cells = 0, my_runs = 0;
+    const int64_t warps = (int64_t)gridDim.x * kDenumWarps;
+    for (int64_t k0 = (blockIdx.x * (int64_t)kDenumWarps + (threadIdx.x >> 5)) * 32; k0 < e.K; k0 += warps * 32) {
+        const int64_t key = k0 + lane;
+        unsigned long long a0 = 0;
+        uint32_t q = 0;
+        if (key < e.K) {
+            a0 = off64[key];
+            q = (uint32_t)(off64[key + 1] >> 32) - (uint32_t)(a0 >> 32);
+            if (MODE == 0 && q == 0) run_cnt[key] = 0;
+        }
+        uint32_t cc[kMaxM] = {};
+        unsigned occupied = __ballot_sync(0xffffffffu, q > 0);
+        if (occupied == 0u) continue;
+#pragma unroll
+        for (int k = 0; k < kMaxM; ++k)
+            if (k < e.m) cc[k] = ((uint32_t)key / e.stride[k]) % e.ncell[k];
+        if (q > 0 && COUNT) {
+            my_sq += (unsigned long long)q * (unsigned long long)q;
+            if (e.symmetric) my_skip += tri_skip((int64_t)q, (int)e.qmax);
+            ++my_cells;
+        }
+        for (; occupied; occupied &= occupied - 1u) {
+            const int src = __ffs(occupied) - 1;
+            const uint32_t k32 = (uint32_t)k0 + (uint32_t)src;
+            const uint32_t cq = __shfl_sync(0xffffffffu, q, src);
+            const unsigned long long ca = __shfl_sync(0xffffffffu, a0, src);
+            uint32_t c[kMaxM];
+#pragma unroll
+            for (int k = 0; k < kMaxM; ++k) c[k] = __shfl_sync(0xffffffffu, cc[k], src);
+            uint32_t last = 0, nlast = 0;
+#pragma unroll
+            for (int k = 0; k < kMaxM; ++k)
+                if (k == mm) {
+                    last = c[k];
+                    nlast = e.ncell[k];
+                }
+            const uint32_t below = last > 0 ? 1u : 0u, above = last + 1 < nlast ? 1u : 0u;
+            const uint32_t r0 = MODE == 1 ? run_off[k32] : MODE == 2 ? k32 * slots : 0u;
+            uint32_t nr = 0;
+            unsigned long long ev = 0;
+            for (int v0 = 0; v0 < nvec; v0 += 32) {
+                const int vi = v0 + lane;
+                // up to two runs of keys [ka, kb]: the neighbours' row, or (zero
+                // vector of a symmetric join) the cell itself and the next
+                uint32_t ka = 0, kb = 0;
+                bool one = false, two = false, mirror = false;
+                if (vi < nvec) {
+                    const uint32_t off = s_off[vi], sign = off >> 12;
+                    bool inside = !(e.symmetric && sign == 2u);
+#pragma unroll
+                    for (int k = 0; k < kMaxM - 1; ++k)
+                        if (k < mm) inside = inside && c[k] + ((off >> (2 * k)) & 3u) - 1u < e.ncell[k];  // (-1 wraps)
+                    const uint32_t base = k32 + (uint32_t)s_delta[vi];
+                    one = inside;
+                    if (e.symmetric && sign == 0u) {
+                        ka = kb = base;
+                        two = inside && above != 0u;
+                    } else {
+                        ka = base - below;
+                        kb = base + above;
+                        mirror = e.symmetric != 0;
+                    }
+                }
+                int32_t a = 0, b = 0, b2 = 0;
+                if (one) {
+                    a = (int32_t)(off64[ka] >> 32);
+                    b = (int32_t)(off64[kb + 1] >> 32);
+                }
+                if (two) b2 = (int32_t)(off64[kb + 2] >> 32);
+                one = one && a < b;
+                two = two && b < b2;
+                const unsigned w1 = __ballot_sync(0xffffffffu, one), w2 = __ballot_sync(0xffffffffu, two);
+                if (FILL) {
+                    const unsigned lt = (1u << lane) - 1u;
+                    uint32_t at = r0 + nr + (uint32_t)__popc(w1 & lt) + (uint32_t)__popc(w2 & lt);
+                    if (one) {
+                        Run rr;
+                        rr.start = a;
+                        rr.end_flags = (uint32_t)b | (mirror ? kMirrorBit : 0u);
+                        runs[at++] = rr;
+                    }
+                    if (two) {
+                        Run rr;
+                        rr.start = b;
+                        rr.end_flags = (uint32_t)b2 | kMirrorBit;
+                        runs[at] = rr;
+                    }
+                }
+                nr += (uint32_t)__popc(w1) + (uint32_t)__popc(w2);
+                if (one) ev += (unsigned long long)(b - a);
+                if (two) ev += (unsigned long long)(b2 - b);
+            }
+            if (FILL) {
+                const uint32_t s0 = (uint32_t)(ca >> 32), it0 = (uint32_t)(ca & 0xFFFFFFFFull);
+                for (uint32_t t = lane; t * (unsigned long long)e.qmax < cq; t += 32) {
+                    Item x;
+                    x.q0 = (int32_t)(s0 + t * e.qmax);
+                    x.q1 = (int32_t)(s0 + min(cq, (t + 1) * e.qmax));
+                    x.r0 = (int32_t)r0;
+                    x.r1 = (int32_t)(r0 + nr);
+                    items[it0 + t] = x;
+                }
+            }
+            if (COUNT) {
+                my_eval += ev * (unsigned long long)cq;
+                if (lane == 0) {
+                    my_runs += nr;
+                    if (MODE == 0) run_cnt[k32] = nr;
+                }
+            }
+        }
+    }
+    if (COUNT) {
+        for (int o = 16; o > 0; o >>= 1) {
+            my_eval += __shfl_down_sync(0xffffffffu, my_eval, o);
+            my_sq += __shfl_down_sync(0xffffffffu, my_sq, o);
+            my_skip += __shfl_down_sync(0xffffffffu, my_skip, o);
+            my_cells += __shfl_down_sync(0xffffffffu, my_cells, o);
+        }
+        if (lane == 0 && my_cells) {
+            atomicAdd(&s_tot[0], my_eval);
+            atomicAdd(&s_tot[1], my_sq);
+            atomicAdd(&s_tot[2], my_skip);
+            atomicAdd(&s_tot[3], my_cells);
+            atomicAdd(&s_tot[4], my_runs);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && s_tot[3]) {
+            atomicAdd(&tot->n_evaluated, s_tot[0]);
+            atomicAdd(&tot->sum_sq, s_tot[1]);
+            atomicAdd(&tot->tri_skip, s_tot[2]);
+            atomicAdd(&tot->n_cells, s_tot[3]);
+            atomicAdd(&tot->n_runs, s_tot[4]);
+        }
+    }
+}
+
+template <int MODE>
+static void launch_denum(const DenseEnum& e, int device, const unsigned long long* off64, uint32_t* run_cnt,
+                         const uint32_t* run_off, Run* runs, Item* items, DenseTotals* tot, uint32_t slots,
+                         cudaStream_t s) {
+    if (e.m >= 4) {
+        const int64_t groups = (e.K + 32 * kDenumWarps - 1) / (32 * kDenumWarps);
+        const unsigned blocks = (unsigned)std::min<int64_t>(groups, (int64_t)device_sm_count(device) * 12);
+        k_denum_warp<MODE><<<blocks, 32 * kDenumWarps, 0, s>>>(e, off64, run_cnt, run_off, runs, items, tot, slots);
+    } else {
+        k_denum<MODE><<<(unsigned)((e.K + 127) / 128), 128, 0, s>>>(e, off64, run_cnt, run_off, runs, items, tot, slots);
+    }
+    note_launch();
+}
+
 // ---------------------------------------------------------------------------
 // host orchestration
 // ---------------------------------------------------------------------------
@@ -1385,7 +1580,6 @@ double tc_c1(int dp, int kernel) {
 struct DensePlan {
     DenseEnum de;
     DenseTotals* dtot;
-    unsigned eb;
     int64_t slots, cells_max, items_cap, runs_cap;
     bool fixed;
 };
@@ -1405,7 +1599,6 @@ static int dense_enum_prepare(Index* ix, int64_t K, int qmax, Scratch& tmp, Dens
     de.K = K;
     SJ_TRY(tmp.alloc(&dp->dtot, 1));
     SJ_CK(cudaMemsetAsync(dp->dtot, 0, sizeof(DenseTotals), s));
-    dp->eb = (unsigned)((K + 127) / 128);
     // runs of a cell: at most 3^(m-1), one more when the self offset splits
     // (symmetric joins)
     int mm = ix->m > 0 ? ix->m - 1 : 0, per = 1;
@@ -1595,9 +1788,8 @@ int build_index(Index* ix, const double* pts) {
                 if (!ix->ev_side[e]) SJ_CK(cudaEventCreateWithFlags(&ix->ev_side[e], cudaEventDisableTiming));
             SJ_CK(cudaEventRecord(ix->ev_side[0], s));
             SJ_CK(cudaStreamWaitEvent(side, ix->ev_side[0], 0));
-            k_denum<2><<<dp.eb, 128, 0, side>>>(dp.de, off64, nullptr, nullptr, ix->runs, ix->items, dp.dtot,
-                                                (uint32_t)dp.slots);
-            note_launch();
+            launch_denum<2>(dp.de, ix->device, off64, nullptr, nullptr, ix->runs, ix->items, dp.dtot,
+                            (uint32_t)dp.slots, side);
             SJ_CK(cudaGetLastError());
             SJ_CK(cudaEventRecord(ix->ev_side[1], side));
             side_join.ev = ix->ev_side[1];
@@ -1644,7 +1836,6 @@ int build_index(Index* ix, const double* pts) {
         // end of the build ----
         const DenseEnum& de = dp.de;
         DenseTotals* dtot = dp.dtot;
-        const unsigned eb = dp.eb;
         const int64_t slots = dp.slots, cells_max = dp.cells_max, items_cap = dp.items_cap;
         int64_t runs_cap = dp.runs_cap;
         uint32_t* run_off = nullptr;  // count pass: K + 1 run offsets
@@ -1659,8 +1850,7 @@ int build_index(Index* ix, const double* pts) {
             uint32_t* run_cnt = nullptr;  // K counts, then K + 1 offsets
             SJ_TRY(tmp.alloc(&run_cnt, (size_t)2 * K + 1));
             run_off = run_cnt + K;
-            k_denum<0><<<eb, 128, 0, s>>>(de, off64, run_cnt, nullptr, nullptr, nullptr, dtot, 0u);
-            note_launch();
+            launch_denum<0>(de, ix->device, off64, run_cnt, nullptr, nullptr, nullptr, dtot, 0u, s);
             SJ_CK(cudaGetLastError());
             SJ_TRY((scan_exclusive<uint32_t, LoadU32>(LoadU32{run_cnt}, run_off, K, true, s)));
             runs_cap = cells_max * slots;
@@ -1671,8 +1861,7 @@ int build_index(Index* ix, const double* pts) {
                 runs_cap = (int64_t)total;
             }
             SJ_TRY(dev_alloc_t(&ix->runs, (size_t)std::max<int64_t>(runs_cap, 1), s));
-            k_denum<1><<<eb, 128, 0, s>>>(de, off64, nullptr, run_off, ix->runs, ix->items, nullptr, 0u);
-            note_launch();
+            launch_denum<1>(de, ix->device, off64, nullptr, run_off, ix->runs, ix->items, nullptr, 0u, s);
             SJ_CK(cudaGetLastError());
         }
         struct Got {
