@@ -70,6 +70,10 @@ __device__ __forceinline__ void dbg_record_pruned(const JoinParams& P, int32_t q
     if (k < P.dbg_cap) P.dbg[k] = make_int4(qs, cs, 0, 1);
 }
 
+// The FP32 filter for sparse indexes (sj_join_f32r.cu).
+bool f32r_preferred(const Index* ix, const JoinParams& p);
+int launch_join_f32r(Index* ix, const JoinParams& p);
+
 JoinParams make_join_params(Index* ix, const JoinOut& out, int emit_dist);
 
 // Bounds checks of the debug build (compiled with -DSJ_DEBUG_BOUNDS): a

@@ -1,0 +1,234 @@
+// The certified FP32 filter for small dimensions (padded d <= 8, without
+// distances) on sparse indexes: cells of one or two points, as when
+// near-duplicates of a large set are sought.
+//
+// Per pair it computes what k_join_f32s does (the same value, thresholds,
+// recheck queue and stage).  That kernel gives a warp one work item at a time:
+// it loads up to 16 queries, takes their bounding box, prefixes the item's runs
+// and then evaluates chunks of 64 candidates.  With 1.4 queries and 31
+// candidates an item those preparations are nearly all of the work (about 800
+// instructions an item), and the box prunes no more than the evaluation itself.
+// Here a warp takes kF32rItems items together: the runs of all of them are
+// prefixed once, and the lanes take consecutive candidates of that list,
+// whichever item they belong to; a lane finds its run among the at most 32
+// that follow the chunk's first one and walks its own item's queries.  Bound by
+// instruction issue.  Measured (1,000,001 uniform 4-D points, 4 neighbours,
+// 692,967 items): 687 / 274 us.
+#include <algorithm>
+#include <atomic>
+
+#include "sj_f32_stage.cuh"
+
+namespace sj {
+
+namespace {
+
+constexpr int kF32rItems = 8;     // items a warp takes at a time
+constexpr int kF32rRuns = 256;    // runs of a group of them (an item has at most kMaxRuns)
+constexpr int kF32rStage = 256;
+constexpr int kF32rWarps = 4;
+static_assert(kMaxRuns <= kF32rRuns, "a group holds at least one item");
+static_assert(2 * kF32rStage <= kStageMax, "a stage flush (entries and mirrors) resolves at most 32 pages");
+
+struct F32rWarp {
+    int32_t rstart[kF32rRuns];     // per run of the group: first sorted position,
+    uint32_t rpre[kF32rRuns + 1];  // prefix of the lengths,
+    uint8_t rmeta[kF32rRuns];      // item of the group | flag << 4 (0 plain, 1 mirrored, 2 self-cell triangle)
+    int2 iq[kF32rItems];           // per item: its queries [x, y)
+    int32_t ipre[kF32rItems + 1];  // prefix of the items' runs in the group
+    int32_t ir0[kF32rItems];       // first run
+    unsigned long long rechecked;  // pairs re-decided in place, queue full (lane 0)
+    int smir;                      // staged entries flagged for a mirrored copy (lane 0)
+    int2 stage[kF32rStage];
+};
+
+template <int DP>
+__global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P) {
+    __shared__ F32rWarp smem[kF32rWarps];
+    const float* __restrict__ Y = static_cast<const float*>(P.y);
+    const float* __restrict__ H = static_cast<const float*>(P.h);
+    const int lane = threadIdx.x & 31;
+    F32rWarp& W = smem[threadIdx.x >> 5];
+    WarpStage st{W.stage, nullptr, 0, 0, kF32rStage};
+    if (lane == 0) {
+        W.rechecked = 0;
+        W.smir = 0;
+    }
+    for (;;) {
+        long long first = 0;
+        if (lane == 0) first = (long long)atomicAdd(&P.counters[0], (unsigned long long)kF32rItems);
+        first = __shfl_sync(0xffffffffu, first, 0);
+        if (first >= P.n_items) break;
+        Item I{0, 0, 0, 0};
+        if (lane < kF32rItems && first + lane < P.n_items) I = P.items[first + lane];
+        if (!SJ_BOUND(P, I.q0 >= 0 && I.q1 <= P.n_points && I.r1 - I.r0 <= kF32rRuns, 51)) I = Item{0, 0, 0, 0};
+        const int have = (int)min((long long)kF32rItems, P.n_items - first);
+        int upto = I.r1 - I.r0;  // inclusive prefix of the items' runs
+#pragma unroll
+        for (int o = 1; o < kF32rItems; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, upto, o);
+            if (lane >= o) upto += u;
+        }
+        for (int j0 = 0, taken = 0; j0 < have;) {  // groups of items whose runs fit
+            const unsigned fit = __ballot_sync(0xffffffffu, lane >= j0 && lane < have && upto - taken <= kF32rRuns);
+            const int nj = __popc(fit);  // (consecutive from j0, at least one)
+            __syncwarp();
+            if (lane >= j0 && lane < j0 + nj) {
+                W.iq[lane - j0] = make_int2(I.q0, I.q1);
+                W.ir0[lane - j0] = I.r0;
+                W.ipre[lane - j0 + 1] = upto - taken;
+            }
+            if (lane == 0) W.ipre[0] = 0;
+            __syncwarp();
+            const int nruns = W.ipre[nj];
+            uint32_t carry = 0;
+            for (int b = 0; b < nruns; b += 32) {
+                const int f = b + lane;
+                uint32_t len = 0;
+                if (f < nruns) {
+                    int j = 0;
+                    while (W.ipre[j + 1] <= f) ++j;
+                    const Run R = P.runs[W.ir0[j] + f - W.ipre[j]];
+                    const bool self = P.tri && !(R.end_flags & kMirrorBit);
+                    const int32_t start = self ? W.iq[j].x : R.start;
+                    W.rstart[f] = start;
+                    W.rmeta[f] = (uint8_t)(j | (self ? 2 : (int)(R.end_flags >> 31)) << 4);
+                    len = (uint32_t)((int32_t)(R.end_flags & ~kMirrorBit) - start);
+                }
+                uint32_t v = len;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t u = __shfl_up_sync(0xffffffffu, v, o);
+                    if (lane >= o) v += u;
+                }
+                if (f < nruns) W.rpre[f + 1] = carry + v;
+                carry += __shfl_sync(0xffffffffu, v, 31);
+            }
+            if (lane == 0) W.rpre[0] = 0;
+            __syncwarp();
+            const uint32_t C = carry;
+            int run0 = 0;  // the run of the chunk's first candidate
+            for (uint32_t v0 = 0; v0 < C; v0 += 32) {
+                const uint32_t v = v0 + (uint32_t)lane;
+                if (W.rpre[run0 + 1] <= v0) ++run0;  // (the last chunk ended with its run)
+                // the last run r with rpre[r] <= v (runs are not empty, so it is
+                // one of the 32 from the first candidate's on)
+                int lo = run0, hi = min(run0 + 31, nruns - 1);
+#pragma unroll
+                for (int k = 0; k < 5; ++k) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    const bool up = W.rpre[mid] <= v;
+                    lo = up ? mid : lo;
+                    hi = up ? hi : mid - 1;
+                }
+                run0 = __shfl_sync(0xffffffffu, lo, 31);
+                const bool valid = v < C;
+                int32_t j = 0, q = 0, qe = 0, cid = 0;
+                int fl = 0;
+                float c[DP], to = INFINITY, ti = INFINITY;
+                if (valid) {
+                    const uint32_t meta = W.rmeta[lo];
+                    const int2 iq = W.iq[meta & 15u];
+                    fl = (int)(meta >> 4);
+                    j = W.rstart[lo] + (int32_t)(v - W.rpre[lo]);
+                    if (!SJ_BOUND(P, j >= 0 && j < P.n_points, 52)) j = 0;
+                    q = iq.x;
+                    qe = fl == 2 ? min(iq.y, j + 1) : iq.y;  // (the triangle: queries up to the candidate)
+                    load_coords<DP>(Y, j, c);
+                    const float4 ax = P.aux[j];
+                    to = ax.x;
+                    ti = ax.y;
+                    cid = __float_as_int(ax.z);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < DP; ++k) c[k] = 0.f;
+                }
+                while (__any_sync(0xffffffffu, q < qe)) {
+                    int nout = 0;
+                    int32_t qid = 0;
+                    bool band = false, mir = false;
+                    if (q < qe) {
+                        float y[DP];
+                        load_coords<DP>(Y, q, y);
+                        float a = H[q];
+#pragma unroll
+                        for (int k = 0; k < DP; ++k) a = __fmaf_rn(y[k], c[k], a);
+                        if (a >= to) {
+                            mir = fl != 0 && q != j;
+                            if (a >= ti) {
+                                nout = mir ? 2 : 1;
+                                qid = P.perm[q];
+                            } else {
+                                band = true;
+                            }
+                        }
+                    }
+                    if (__any_sync(0xffffffffu, band)) {
+                        const bool queued = band_push(P, lane, band, q, j, mir);
+                        const bool here = band && !queued;
+                        const unsigned inplace = __ballot_sync(0xffffffffu, here);
+                        if (lane == 0 && inplace) W.rechecked += (unsigned long long)__popc(inplace);
+                        if (here && direct_sq(P.xs + (int64_t)q * P.dp, P.xs + (int64_t)j * P.dp, P.d) <= P.e2) {
+                            nout = mir ? 2 : 1;
+                            qid = P.perm[q];
+                        }
+                    }
+                    f32s_emit<false>(W, st, P, lane, nout, qid, cid);
+                    ++q;
+                }
+            }
+            j0 += nj;
+            taken = __shfl_sync(0xffffffffu, upto, j0 - 1);
+        }
+    }
+    f32s_flush<false>(W, st, P, lane);
+    if (lane == 0 && W.rechecked) atomicAdd(&P.counters[2], W.rechecked);
+}
+
+template <int DP>
+int launch_f32r_d(Index* ix, const JoinParams& p) {
+    auto kern = k_join_f32r<DP>;
+    static std::atomic<int> cached{0};  // resident CTAs per SM (a property of the kernel)
+    int per_sm = cached.load(std::memory_order_relaxed);
+    if (per_sm == 0) {
+        SJ_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kF32rWarps, 0));
+        if (per_sm < 1) per_sm = 1;
+        cached.store(per_sm, std::memory_order_relaxed);
+    }
+    const long long need = (ix->n_items + kF32rItems * kF32rWarps - 1) / (kF32rItems * kF32rWarps);
+    const long long blocks = std::max<long long>(1, std::min<long long>(need, (long long)device_sm_count(ix->device) * per_sm));
+    kern<<<(unsigned)blocks, 32 * kF32rWarps, 0, ix->stream>>>(p);
+    note_launch();
+    SJ_CK(cudaGetLastError());
+    return SJ_OK;
+}
+
+}  // namespace
+
+// Taken for single joins when cells are sparse: fewer than 2.5 queries an item
+// (1.9 for padded d = 8, whose candidates cost more to load) and, against a few
+// crowded cells among many single ones, fewer than 160 (300) evaluations an
+// item.  Both kernels, us, by queries an item: uniform 4-D 1.1 754 / 155, 1.4
+// 667 / 274, 2.0 540 / 352, 3.2 419 / 475; 3-D 1.6 283 / 88, 3.9 156 / 151; 2-D
+// 1.8 375 / 164, 2.8 286 / 210, 5.1 195 / 279; 5-D 1.8 323 / 245, 3.8 266 / 500;
+// 6-D 1.2 336 / 189, 1.8 348 / 382; clusters over noise, 3-D 1.6 464 / 333, 2.7
+// 387 / 927.  (Batched joins and the filter's recording mode keep k_join_f32s.)
+bool f32r_preferred(const Index* ix, const JoinParams& p) {
+    if (p.batch || p.dbg || ix->n_cells <= 0) return false;
+    const double items = (double)ix->n_cells + (double)ix->n / kQMax;
+    return ix->dp <= 4 ? (double)ix->n < 2.5 * items && (double)ix->n_evaluated < 160.0 * items
+                       : (double)ix->n < 1.9 * items && (double)ix->n_evaluated < 300.0 * items;
+}
+
+int launch_join_f32r(Index* ix, const JoinParams& p) {
+    switch (ix->dp) {
+        case 2: return launch_f32r_d<2>(ix, p);
+        case 4: return launch_f32r_d<4>(ix, p);
+        case 8: return launch_f32r_d<8>(ix, p);
+        default:
+            set_error("no small-d FP32 kernel for padded dimension %d", ix->dp);
+            return SJ_ERR_UNSUPPORTED;
+    }
+}
+
+}  // namespace sj
