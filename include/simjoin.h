@@ -191,8 +191,8 @@ typedef struct sj_result {
     int64_t n_evaluated;      /* pair evaluations performed by the kernel: the
                                  index's scheduled evaluations less those the
                                  FP32 filter's bounding-box prune (padded
-                                 d <= 8) removed; batched results report the
-                                 scheduled evaluations */
+                                 d <= 8) removed; batched results and the FP64
+                                 tile report the scheduled evaluations */
     int64_t n_rechecked;      /* pairs the kernel's certified bound left open,
                                  re-decided by the direct form (behind a
                                  tensor-core filter in binary32 with a bound of

@@ -549,6 +549,19 @@ void pack_coefficients(double eps, double pbound, double delta, double u_t, int 
     pp->refine_in = si_r > 0 && si >= ldexp(1.0, -60) ? down(si * (1.0 - rel)) : -1.f;
 }
 
+// Radius^2 of the bounding-box prune in front of the FP64 tile, whose kernel
+// coordinates are rounded to binary32 for that test: each is then off by at
+// most 2^-24 R beside the delta of the binary64 ones, which u_T = 2^-24 covers,
+// so this is the binary32 filters' S_o without a scale.  +inf (no prune) for
+// an extent whose coordinates binary32 cannot hold; where the squares
+// underflow the test's rounded-down bound is 0 and keeps everything.
+static float fp64_prune_r2(double eps, double rmax, int d) {
+    if (!(rmax < 1e15)) return INFINITY;
+    PackParams pp{};
+    pack_coefficients(eps, 0.0, 1.02 * ldexp(1.0, -24) * rmax, ldexp(1.0, -24), d, d, &pp);
+    return pp.prune_r2f;
+}
+
 // The two thresholds of a point with computed norm pc, one fma each, rounded
 // outward (see pack_coefficients).
 __device__ __forceinline__ float pack_thr_out(const PackParams& pp, float pc) {
@@ -1735,7 +1748,7 @@ int build_index(Index* ix, const double* pts) {
     hp.scale = scale;
     ix->kscale = scale;
     pack_coefficients(ix->eps * scale, pbound * scale * scale, delta * scale, u_t, d, ix->dp, &hp, c1);
-    ix->prune_r2 = hp.prune_r2f;
+    ix->prune_r2 = use_f32 ? hp.prune_r2f : fp64_prune_r2(ix->eps, rmax, d);
     ix->refine_out = hp.refine_out;
     ix->refine_in = hp.refine_in;
 

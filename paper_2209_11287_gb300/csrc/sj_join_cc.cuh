@@ -55,7 +55,74 @@ struct CcWarpSmem {
     int2 stage[kStage];
     double sdist[EMIT ? kStage : 1];
     double scq[DP >= 16 ? kQMax : 1];  // short-circuit: each query's w
+    // d <= 8: candidates kept by the bounding-box prune (position, run flag),
+    // and the box of the item's queries
+    static constexpr uint32_t RING = 32 * TC - 1 + 64 <= 128 ? 128 : 256;
+    int32_t ring_j[DP <= 8 ? RING : 1];
+    uint8_t ring_f[DP <= 8 ? RING : 1];
+    float blo[DP <= 8 ? DP : 1], bhi[DP <= 8 ? DP : 1];
 };
+
+// Compaction step of the prune, d <= 8: candidates [v0, v0 + 64) of the item,
+// two a lane, against the box of its queries; the kept ones follow the ring's
+// `cnt` entries from `head`.  The same lossless test as k_join_f32s
+// (f32s_gather: a lower bound of the squared distance to the box, every
+// operation rounded down, against the radius behind the certified "out"
+// threshold), here in front of the tiles with distances and the FP64 tile.
+// The latter's binary64 coordinates are rounded to binary32 for it, which its
+// radius allows for (fp64_prune_r2).  `r` is the lane's run cursor.
+// A radius of +inf keeps everything.  Returns the candidates dropped.  Measured,
+// FP64 tile with distances (200,000 uniform 4-D points, 64 neighbours, 9 queries
+// an item; FP64 pipe): 705 us over all candidates, 495 us behind the prune.
+template <typename T, int DP, int TC, bool EMIT, int RUNS>
+__device__ __forceinline__ uint32_t cc_gather(CcWarpSmem<T, DP, TC, EMIT, RUNS>& W, const JoinParams& P, float r2,
+                                              uint32_t C, uint32_t v0, int lane, int& r, uint32_t head, uint32_t& cnt) {
+    constexpr uint32_t RING = CcWarpSmem<T, DP, TC, EMIT, RUNS>::RING;
+    const T* __restrict__ Y = static_cast<const T*>(P.y);
+    ItemSmem<T, DP, RUNS>& S = W.it;
+    int32_t jj[2];
+    uint32_t f[2];
+    bool keep[2], test[2];
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        const uint32_t v = v0 + (uint32_t)(32 * g + lane);
+        jj[g] = 0;
+        f[g] = 0;
+        keep[g] = v < C;
+        if (v < C) {
+            while (S.rpre[r + 1] <= v) ++r;
+            jj[g] = S.rstart[r] + (int32_t)(v - S.rpre[r]);
+            if (!SJ_BOUND(P, jj[g] >= 0 && jj[g] < P.n_points && r < RUNS, 21)) jj[g] = 0;
+            f[g] = S.rmir[r];
+        }
+        test[g] = keep[g] && f[g] != 2u && r2 < INFINITY;
+    }
+    float c[2][DP];
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+#pragma unroll
+        for (int k = 0; k < DP; ++k) c[g][k] = test[g] ? (float)Y[(int64_t)jj[g] * DP + k] : 0.f;
+    uint32_t kept = 0;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        float lb = 0.f;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) {
+            const float gap = fmaxf(fmaxf(__fsub_rd(W.blo[k], c[g][k]), __fsub_rd(c[g][k], W.bhi[k])), 0.f);
+            lb = __fmaf_rd(gap, gap, lb);
+        }
+        if (test[g] && lb > r2) keep[g] = false;
+        const unsigned m = __ballot_sync(0xffffffffu, keep[g]);
+        if (keep[g]) {
+            const uint32_t e = (head + cnt + kept + (uint32_t)__popc(m & ((1u << lane) - 1u))) & (RING - 1u);
+            W.ring_j[e] = jj[g];
+            W.ring_f[e] = (uint8_t)f[g];
+        }
+        kept += (uint32_t)__popc(m);
+    }
+    cnt += kept;
+    return min(64u, C - v0) - kept;
+}
 
 // Maybe-in bitmasks of TC candidates against all queries of the item, d <= 8:
 // the threshold test follows each query's fma chain.
@@ -199,14 +266,12 @@ __device__ __forceinline__ void emit_direct(WarpStage& st, const JoinParams& P, 
 }
 
 // Minimum resident CTAs per SM requested from the register allocator, and
-// candidates per lane, of the FP32 small-d tile (d <= 8): it is
-// latency-bound, so it runs with 2 candidates per lane and 9 CTAs of 4
-// warps per SM (at most 56 registers).  Measured on the uniform 4-D
-// workload (2M points), tile-kernel time: 2 candidates x 9 CTAs 1.196 ms,
-// 2 x 10 1.218, 2 x 8 1.235, 2 x 12 1.521, 2 x 16 1.781, 4 x 8 1.323,
-// 4 x 7 1.372, 4 x 6 1.428.  Compile-time tuning constants.
+// candidates per lane, of the FP32 small-d tile with distances (d <= 8).
+// Measured behind the bounding-box prune (200,003 uniform 3-D points, 48
+// neighbours), tile-kernel time: 9 CTAs (56 registers, spills) 156 us, 8 152,
+// 7 150; without the prune 155.  Compile-time tuning constants.
 #ifndef SJ_CC_F32_MIN_BLOCKS
-#define SJ_CC_F32_MIN_BLOCKS 9
+#define SJ_CC_F32_MIN_BLOCKS 7
 #endif
 #ifndef SJ_CC_TC_SMALL_D
 #define SJ_CC_TC_SMALL_D 2
@@ -232,7 +297,7 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
     ItemSmem<T, DP, RUNS>& S = W.it;
     WarpStage st{W.stage, EMIT ? W.sdist : nullptr, 0, 0};
     BandQ bq{0, 0};
-    unsigned long long rechecked = 0;
+    unsigned long long rechecked = 0, pruned = 0;  // (pruned: the same in all lanes)
 
     long long next = 0;
     if (lane == 0) next = (long long)atomicAdd(&P.counters[0], 1ull);
@@ -254,7 +319,44 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
             }
         }
 
-        for (uint32_t base = 0; base < C; base += (uint32_t)SLOTS) {
+        float box_r2 = INFINITY;
+        if constexpr (FUSED) {  // the box of the queries (32 is a multiple of DP: a lane keeps to one dim)
+            // (a batched FP64 join has no radius that allows for the rounding)
+            box_r2 = std::is_same<T, double>::value && P.batch ? INFINITY : R.r2;
+            float bmin = INFINITY, bmax = -INFINITY;
+            for (int i = lane; i < Q * DP; i += 32) {
+                const float v = (float)S.qy[i / DP][i % DP];
+                bmin = fminf(bmin, v);
+                bmax = fmaxf(bmax, v);
+            }
+#pragma unroll
+            for (int o = DP; o < 32; o <<= 1) {
+                bmin = fminf(bmin, __shfl_xor_sync(0xffffffffu, bmin, o));
+                bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
+            }
+            if (lane < DP) {
+                W.blo[lane] = bmin;
+                W.bhi[lane] = bmax;
+            }
+            __syncwarp();
+        }
+        int run = 0;
+        uint32_t head = 0, cnt = 0, v0 = 0;  // the ring (d <= 8); candidates gathered
+        for (uint32_t base = 0;;) {
+            uint32_t ns;  // candidates of this chunk
+            if constexpr (FUSED) {
+                while (v0 < C && cnt < (uint32_t)SLOTS) {
+                    const uint32_t out = cc_gather<T, DP, TC, EMIT, RUNS>(W, P, box_r2, C, v0, lane, run, head, cnt);
+                    if constexpr (std::is_same<T, float>::value) pruned += (unsigned long long)out * (unsigned long long)Q;
+                    v0 += 64u;
+                }
+                if (cnt == 0) break;
+                ns = min(cnt, (uint32_t)SLOTS);
+                __syncwarp();
+            } else {
+                if (base >= C) break;
+                ns = min(C - base, (uint32_t)SLOTS);
+            }
             int32_t j[TC];
             bool valid[TC];
             uint32_t tri_mask[TC];
@@ -262,16 +364,21 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
 #pragma unroll
             for (int t = 0; t < TC; ++t) {
                 const int slot = t * 32 + lane;
-                const uint32_t v = base + (uint32_t)slot;
-                valid[t] = v < C;
+                valid[t] = (uint32_t)slot < ns;
                 j[t] = 0;
                 tri_mask[t] = 0xFFFFFFFFu;
                 to[t] = T(INFINITY);  // an empty slot is never maybe-in
                 ti[t] = T(INFINITY);
                 if (valid[t]) {
                     uint8_t fl;
-                    j[t] = map_candidate_flag<T, DP>(S, nr, v, fl);
-                    if (!SJ_BOUND(P, j[t] >= 0 && j[t] < P.n_points, 21)) j[t] = 0;
+                    if constexpr (FUSED) {
+                        const uint32_t e = (head + (uint32_t)slot) & (CcWarpSmem<T, DP, TC, EMIT, RUNS>::RING - 1u);
+                        j[t] = W.ring_j[e];
+                        fl = W.ring_f[e];
+                    } else {
+                        j[t] = map_candidate_flag<T, DP>(S, nr, base + (uint32_t)slot, fl);
+                        if (!SJ_BOUND(P, j[t] >= 0 && j[t] < P.n_points, 21)) j[t] = 0;
+                    }
                     to[t] = TO[j[t]];
                     ti[t] = TI[j[t]];
                     if constexpr (EMIT) W.cj[slot] = j[t];
@@ -418,11 +525,19 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
             __syncwarp();
             }
             }
+            if constexpr (FUSED) {
+                head = (head + ns) & (CcWarpSmem<T, DP, TC, EMIT, RUNS>::RING - 1u);
+                cnt -= ns;
+                __syncwarp();
+            } else {
+                base += (uint32_t)SLOTS;
+            }
         }
         __syncwarp();
     }
     band_q_close(bq, P, lane);
     stage_flush(st, P, lane);
+    if (lane == 0 && pruned) atomicAdd(&P.counters[6], pruned);
     for (int o = 16; o > 0; o >>= 1) rechecked += __shfl_down_sync(0xffffffffu, rechecked, o);
     if (lane == 0 && rechecked) atomicAdd(&P.counters[2], rechecked);
 }
