@@ -20,36 +20,38 @@
 // One persistent CTA per SM, warp-specialised:
 //   warp 0      tiles: takes work items from the queue and cuts the item's
 //               candidate runs into tiles (128 rows = 16 8-row groups), per
-//               tile the rows' metadata and the copies that bring them;
+//               tile the rows' ranges and the copies that bring them, two
+//               tiles at a time;
 //   warp 1      MMA issuer (one thread): K/16 MMAs per tile into one of two
 //               TMEM accumulators (128 lanes x N columns), committed to the
 //               stage and accumulator barriers;
 //   warp 2      copies (one thread): the item's query tile (MMA B, N <= 256
 //               queries, 8-row groups from an 8-aligned start; the next
 //               item's while this one runs, where shared memory allows) and
-//               the candidate tiles (MMA A) in K-slices of 64, bulk copies
-//               completing on mbarriers;
-//   warps 3..   epilogue (16 or 8 warps): each thread owns one candidate row
-//               (its TMEM lane) and a share of its N accumulators (EPI / 4
-//               warps per lane quarter, interleaved 32-column chunks): a max
-//               over the chunk against the row's threshold first (hits are
-//               rare), then column masks of the maybe-in and the certain ones
-//               and a record.
-// What bounds it: at K = 64 the epilogue's instruction issue (57% of the issue
-// slots, about 330 instructions a warp and tile), so it holds only what has to
-// happen while the accumulator is there, and an accumulator is released as
-// soon as its last columns are in registers.  Emitting the pairs here (ids,
-// compaction, pages, recheck queue, by half-empty warps) made every warp wait
-// for that serial code in turn.  Resolving the rows of a tile and its copies
-// used to be one warp's work (about 1,100 cycles a tile, 1,900 with many runs,
-// slower than the MMA's 512); the two halves now overlap.  16 epilogue warps
-// with one chunk in registers each (96 registers) against 8 warps with two
-// (150): 1.99 / 2.34 ms (2^17 x 16-D without an index), 2.84 / 3.14 (500,000 x
-// 16-D mixture), 4.07 / 3.83 (150,000 x 64-D): at K = 208 the MMA binds (the
-// shared-memory reads of its operands, 12 KB per 128 cycles) and more warps
-// only compete with it, so the line lies between K = 112 and 208.  Tile kernel
-// before / now: 2.85 / 1.99 ms, 5.21 / 2.84 ms, and 7.50 / 6.89 ms at 200,000 x
-// 64-D.
+//               the candidate tiles (MMA A) in K-slices of 64, one or two a
+//               pipeline stage, bulk copies completing on mbarriers;
+//   warp 3      rows: position, flag and thresholds of the tile's rows, fetched
+//               a tile ahead, into shared memory beside the accumulator;
+//   warps 4..   epilogue (16 warps): each thread owns one candidate row (its
+//               TMEM lane) and a quarter of its N accumulators (interleaved
+//               32-column chunks): a max over the chunk against the row's
+//               threshold first (hits are rare), then column masks of the
+//               maybe-in and the certain ones and a record.
+// What bounds it: at K = 208 the MMA (2.2 PFLOP/s of it when the epilogue is
+// left out, 1.97 with it); at K = 64 the epilogue's instruction issue, so it holds
+// only what has to happen while the accumulator is there, an accumulator is
+// released as soon as its last columns are in registers, and a tile costs an
+// epilogue warp one wait and one 16-byte read.  Each role's code is a short
+// loop of its own: waits and copies of one thread cost some 250 cycles a stage
+// beside 16 other warps, so serial work per slice, not bandwidth, kept the MMA
+// waiting (one producer warp: 700 cycles a slice and up to 1,900 a tile of many
+// runs; the 64-D workload was at half the MMA's rate with any number of stages,
+// any copy size and half the MMAs left out).  Tile kernel with what follows it,
+// at the outset / emission moved to k_resolve / roles split: 2^17 x 16-D without
+// an index 2.93 / 2.06 / 1.71 ms, 500,000 x 16-D mixture 5.92 / 3.21 / 2.64,
+// 200,000 x 64-D 8.09 / 7.10 / 4.15.  8 epilogue warps with two chunks in
+// registers each instead of 16 with one: 2.40 / 3.48 / 2.83 (150,000 x 64-D,
+// against 2.06 / 3.17 / 2.64).
 // A symmetric join evaluates only the triangle of each self cell: the self
 // run starts at the item's first query and pairs below the diagonal are
 // masked.  Every wait is bounded; on expiry the CTA stops issuing work,
@@ -65,11 +67,8 @@ constexpr int kTcM = 128;             // candidate rows per tile (TMEM lanes)
 constexpr int kTcG = kTcM / 8;        // 8-row groups per tile
 constexpr int kKS = 64;               // K per pipeline slice
 constexpr int kMetaDepth = 8;         // tiles of row metadata in flight
-// Epilogue warps (EPI / 4 per TMEM lane quarter, splitting the columns) and
-// the 32-column chunks a warp holds at a time.
-constexpr int tc_epi(int kp) { return kp <= 112 ? 16 : 8; }
-constexpr int tc_chunks(int kp) { return kp <= 112 ? 1 : 2; }
-constexpr int tc_threads(int kp) { return 96 + 32 * tc_epi(kp); }  // tile, MMA and copy warps, epilogue
+constexpr int kTcEpi = 16;            // epilogue warps, four per TMEM lane quarter, splitting the columns
+constexpr int kTcThreads = 128 + 32 * kTcEpi;  // tile, MMA, copy and row warps, epilogue
 constexpr long long kTcSpin = 1 << 22;  // bound on barrier polls per wait
 
 struct TcParams {
@@ -84,7 +83,13 @@ template <int KP>
 struct TcShape {
     static constexpr int NMAX = tc_nmax(KP);
     static constexpr int SLICES = (KP + kKS - 1) / kKS;
-    static constexpr int A_STAGE = kTcM * kKS * 2;  // bytes
+    // K-slices of a pipeline stage: the copy and the MMA thread pay a wait and
+    // an arrival (about 250 cycles) a stage, so two where a tile has several
+    static constexpr int GS = SLICES > 1 ? 2 : 1;
+    static constexpr int GROUPS = (SLICES + GS - 1) / GS;
+    static constexpr int A_SLICE = kTcM * kKS * 2;  // bytes
+    static constexpr int A_STAGE = GS * A_SLICE;
+    static constexpr int slice_k(int sl) { return KP - sl * kKS < kKS ? KP - sl * kKS : kKS; }
     static constexpr int B_BYTES = NMAX * KP * 2;
     static constexpr int NB = KP <= 112 ? 2 : 1;  // query tiles in flight (as shared memory allows)
 };
@@ -109,7 +114,7 @@ struct TcMeta {
 
 template <int KP>
 struct TcSmem {
-    static constexpr int EPI = tc_epi(KP);
+    static constexpr int EPI = kTcEpi;
     static_assert(EPI % 4 == 0, "epilogue warps come in whole warpgroups");
     static constexpr int MAX_STAGES = 8;
     uint64_t a_full[MAX_STAGES], a_empty[MAX_STAGES];
@@ -122,6 +127,9 @@ struct TcSmem {
     int abort;
     TcItem items[2];
     TcMeta meta[kMetaDepth];
+    // per accumulator, what its epilogue needs of each row: candidate position,
+    // flag, and the negated thresholds as floats (-inf: no candidate)
+    int4 rows[2][kTcM];
     int32_t rgp[kMaxRuns];  // tile warp: per run of the item, its first group's number in the item
     int32_t rlo[kMaxRuns], rhi[kMaxRuns];
     uint8_t rfl[kMaxRuns];
@@ -144,11 +152,14 @@ constexpr size_t tc_smem_bytes() {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Shared-memory matrix descriptor: K-major, no swizzle.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+// Shared-memory matrix descriptor: K-major core matrices (8 rows x 16 bytes,
+// contiguous along K), 8-row groups `sbo` bytes apart, no swizzle; a K step of 16
+// advances the address by 256 bytes.  (The 128-byte swizzled layout ran at the
+// same speed: 2.38 / 2.34 ms for 150,000 x 64-D.)
+__device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t sbo) {
     uint64_t d = 0;
     d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
+    d |= (uint64_t)(128 >> 4) << 16;
     d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
     d |= (uint64_t)1 << 46;  // descriptor version bits 46-48 = 0b001
     return d;
@@ -161,6 +172,13 @@ __host__ __device__ constexpr uint32_t umma_idesc(int m, int n, uint32_t ab_bf16
            ((uint32_t)(m >> 4) << 24);
 }
 
+// One lane of a converged warp (the compiler then knows that one thread runs
+// the branch, and keeps the operands of copies and MMAs in uniform registers).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+    return p != 0u;
+}
 __device__ __forceinline__ void bar_init(uint64_t* b, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
 }
@@ -199,10 +217,10 @@ __device__ __forceinline__ bool bar_wait_warp(uint64_t* b, uint32_t parity, vola
     return __all_sync(0xffffffffu, bar_wait(b, parity, abort));
 }
 // Bulk copy global -> shared completing on an mbarrier.
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(bar)
         : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
@@ -303,11 +321,12 @@ __device__ __forceinline__ void tc_record(TcRecords& rec, const JoinParams& P, i
 // DBG: the recording instantiation of the filter dump (a test aid; the join
 // kernels proper carry none of its code).
 template <int KP, bool DBG>
-__global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcParams T) {
+__global__ void __launch_bounds__(kTcThreads, 1) k_join_tc(JoinParams P, TcParams T) {
     using SH = TcShape<KP>;
     using SM = TcSmem<KP>;
     constexpr int STAGES = tc_stages<KP>();
     static_assert(STAGES >= 2, "at least two operand stages");
+    static_assert(kTcG == 16, "the tile warp resolves two tiles of 16 groups at a time");
     constexpr int NMAX = SH::NMAX;
     extern __shared__ unsigned char dsm_raw[];
     unsigned char* dsm = reinterpret_cast<unsigned char*>(((uintptr_t)dsm_raw + 1023) & ~(uintptr_t)1023);
@@ -326,13 +345,13 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
             bar_init(&S.b_full[i], 1);
             bar_init(&S.b_empty[i], 1);
             bar_init(&S.item_full[i], 1);
-            bar_init(&S.item_empty[i], 2 + SM::EPI);  // the MMA and copy threads and the epilogue warps
-            bar_init(&S.acc_full[i], 1);
+            bar_init(&S.item_empty[i], 3 + SM::EPI);  // the MMA and copy threads, the row and epilogue warps
+            bar_init(&S.acc_full[i], 2);              // the MMAs are done, the rows written
             bar_init(&S.acc_empty[i], SM::EPI);
         }
         for (int i = 0; i < kMetaDepth; ++i) {
             bar_init(&S.meta_full[i], 1);
-            bar_init(&S.meta_empty[i], 1 + SM::EPI);  // the copy thread and the epilogue warps
+            bar_init(&S.meta_empty[i], 2);  // the copy thread and the row warp
         }
         bar_init(&S.drain, 1);
         S.abort = 0;
@@ -406,11 +425,11 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
             if (it >= P.n_items) break;
             if (++it_i == 2) it_i = 0, it_ph ^= 1u;
             bool bail = false;
-            for (int t = 0; t < ntiles; ++t) {
-                // this lane's group of the tile
-                const int j = t * kTcG + lane;
+            for (int t0 = 0; t0 < ntiles && !bail; t0 += 2) {
+                // this lane's group, of tile t0 (lanes 0 .. 15) or t0 + 1
+                const int j = t0 * kTcG + lane;
                 int4 g = make_int4(-8, 0, 0, 0);
-                if (lane < kTcG && j < ngroups) {
+                if (j < ngroups) {
                     int lo = 0, hi = nr - 1;  // last run whose prefix is <= j
                     while (lo < hi) {
                         const int mid = (lo + hi + 1) >> 1;
@@ -421,28 +440,36 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
                     }
                     g = make_int4((S.rlo[lo] & ~7) + 8 * (j - S.rgp[lo]), S.rlo[lo], S.rhi[lo], S.rfl[lo]);
                 }
-                const int cnt = ngroups - t * kTcG < kTcG ? ngroups - t * kTcG : kTcG;
-                // runs of consecutive groups: their first lanes
+                // runs of consecutive groups in a tile: their first lanes
                 const int32_t gprev = __shfl_up_sync(0xffffffffu, g.x, 1);
-                const bool first = lane < cnt && (lane == 0 || g.x != gprev + 8);
+                const bool first = j < ngroups && ((lane & (kTcG - 1)) == 0 || g.x != gprev + 8);
                 const uint32_t firsts = __ballot_sync(0xffffffffu, first);
-                const uint32_t later = firsts & ~((2u << lane) - 1u);
-                const int seg_end = later ? __ffs(later) - 1 : cnt;
-                if (!bar_wait_warp(&S.meta_empty[m_i], m_ph ^ 1u, abort)) {
-                    bail = true;
-                    break;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (t0 + u >= ntiles) break;
+                    const int cnt = min(ngroups - (t0 + u) * kTcG, kTcG), l = lane - u * kTcG;
+                    const uint32_t mine = (firsts >> (u * kTcG)) & 0xFFFFu;
+                    if (!bar_wait_warp(&S.meta_empty[m_i], m_ph ^ 1u, abort)) {
+                        bail = true;
+                        break;
+                    }
+                    TcMeta& M = S.meta[m_i];
+                    if (l >= 0 && l < kTcG) {
+                        M.g[l] = g;
+                        if (first) {
+                            const uint32_t later = mine & ~((2u << l) - 1u);
+                            M.seg[__popc(mine & ((1u << l) - 1u))] =
+                                make_int4(l, (later ? __ffs(later) - 1 : cnt) - l, g.x >> 3, 0);
+                        }
+                    }
+                    if (lane == 0) {
+                        M.nseg = __popc(mine);
+                        M.cnt = cnt;
+                    }
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(&S.meta_full[m_i]);
+                    if (++m_i == kMetaDepth) m_i = 0, m_ph ^= 1u;
                 }
-                TcMeta& M = S.meta[m_i];
-                if (lane < kTcG) M.g[lane] = g;
-                if (first)
-                    M.seg[__popc(firsts & ((1u << lane) - 1u))] = make_int4(lane, seg_end - lane, g.x >> 3, 0);
-                if (lane == 0) {
-                    M.nseg = __popc(firsts);
-                    M.cnt = cnt;
-                }
-                __syncwarp();
-                if (lane == 0) bar_arrive(&S.meta_full[m_i]);
-                if (++m_i == kMetaDepth) m_i = 0, m_ph ^= 1u;
             }
             if (bail) break;
         }
@@ -450,7 +477,7 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
         // ------------------------------------------------------------ copies
         // One thread: per item the query tile, per tile and K-slice one bulk
         // copy for each run of consecutive groups.
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t a_i = 0, a_ph = 0, m_i = 0, m_ph = 0, it_i = 0, it_ph = 0, b_i = 0, b_ph = 0;
             // stages and query tiles armed so far, and the parity of the last arming
             uint32_t armed_a = 0, par_a = 0, armed_b = 0, par_b = 0;
@@ -471,8 +498,8 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
                     const int ks = KP - sl * kKS < kKS ? KP - sl * kKS : kKS;
                     const __nv_bfloat16* src =
                         T.rows_b + (long long)sl * kKS * T.nrows + (long long)(X.qa >> 3) * ks * 8;
-                    bulk_g2s(sB + (size_t)b_i * SH::B_BYTES + (size_t)NMAX * 2 * kKS * sl, src, gq * (uint32_t)ks * 16u,
-                             &S.b_full[b_i]);
+                    bulk_g2s(smem_u32(sB) + b_i * (uint32_t)SH::B_BYTES + (uint32_t)(NMAX * 2 * kKS * sl), src,
+                             gq * (uint32_t)ks * 16u, smem_u32(&S.b_full[b_i]));
                 }
                 if (++b_i == SH::NB) b_i = 0, b_ph ^= 1u;
                 for (int t = 0; t < X.ntiles && !bail; ++t) {
@@ -482,21 +509,32 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
                     }
                     const TcMeta& M = S.meta[m_i];
                     const int nseg = M.nseg, cnt = M.cnt;
-                    for (int sl = 0; sl < SH::SLICES; ++sl) {
-                        const int ks = KP - sl * kKS < kKS ? KP - sl * kKS : kKS;
+#pragma unroll 1
+                    for (int g = 0; g < SH::GROUPS; ++g) {
                         if (!bar_wait(&S.a_empty[a_i], a_ph ^ 1u, abort)) {
                             bail = true;
                             break;
                         }
-                        bar_arrive_tx(&S.a_full[a_i], (uint32_t)cnt * ks * 16u);
+                        const int k0 = g * SH::GS * kKS, gk = KP - k0 < SH::GS * kKS ? KP - k0 : SH::GS * kKS;
+                        bar_arrive_tx(&S.a_full[a_i], (uint32_t)(cnt * gk) * 16u);
                         armed_a |= 1u << a_i;
                         par_a = (par_a & ~(1u << a_i)) | (a_ph << a_i);
-                        unsigned char* dst = sA + (size_t)a_i * SH::A_STAGE;
-                        const __nv_bfloat16* src = T.rows_a + (long long)sl * kKS * T.nrows;
+                        const uint32_t dst = smem_u32(sA) + a_i * (uint32_t)SH::A_STAGE, bar = smem_u32(&S.a_full[a_i]);
+                        const char* src = reinterpret_cast<const char*>(T.rows_a) + 2 * k0 * T.nrows;
+#pragma unroll 1
                         for (int k = 0; k < nseg; ++k) {
                             const int4 e = M.seg[k];
-                            bulk_g2s(dst + (size_t)e.x * ks * 16, src + (long long)e.z * ks * 8,
-                                     (uint32_t)e.y * ks * 16u, &S.a_full[a_i]);
+                            uint32_t to = dst;
+                            const char* from = src;
+#pragma unroll
+                            for (int u = 0; u < SH::GS; ++u) {
+                                const int left = gk - u * kKS, ks16 = (left < kKS ? left : kKS) * 16;  // bytes a group
+                                if (left > 0)
+                                    bulk_g2s(to + (uint32_t)(e.x * ks16), from + (long long)e.z * ks16,
+                                             (uint32_t)(e.y * ks16), bar);
+                                to += (uint32_t)SH::A_SLICE;
+                                from += 2 * kKS * T.nrows;
+                            }
                         }
                         if (++a_i == STAGES) a_i = 0, a_ph ^= 1u;
                     }
@@ -518,7 +556,7 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             uint32_t a_i = 0, a_ph = 0, it_i = 0, it_ph = 0, b_i = 0, b_ph = 0, acc = 0, acc_ph = 0;
             bool issued = false;
             for (;;) {
@@ -535,23 +573,32 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;");
                     const uint32_t dt = tmem + acc * NMAX;
-                    for (int sl = 0; sl < SH::SLICES; ++sl) {
-                        const int ks = KP - sl * kKS < kKS ? KP - sl * kKS : kKS;
+                    // (unrolled: the descriptors are an address and constants,
+                    // so a K step is issued in a few cycles)
+#pragma unroll
+                    for (int g = 0; g < SH::GROUPS; ++g) {
                         if (!bar_wait(&S.a_full[a_i], a_ph, abort)) {
                             fail = true;
                             break;
                         }
                         asm volatile("tcgen05.fence::after_thread_sync;");
-                        const uint32_t a0 = smem_u32(sA + (size_t)a_i * SH::A_STAGE);
-                        const uint32_t b0 = smem_u32(sB + (size_t)b_i * SH::B_BYTES + (size_t)NMAX * 2 * kKS * sl);
-                        for (int kk = 0; kk < ks / 16; ++kk) {
-                            const uint64_t ad = umma_desc(a0 + kk * 256, 128, (uint32_t)ks * 16u);
-                            const uint64_t bd = umma_desc(b0 + kk * 256, 128, (uint32_t)ks * 16u);
-                            const uint32_t accum = (sl > 0 || kk > 0) ? 1u : 0u;
-                            asm volatile(
-                                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dt),
-                                "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
+                        const uint32_t a0 = smem_u32(sA) + a_i * (uint32_t)SH::A_STAGE;
+                        const uint32_t b0 = smem_u32(sB) + b_i * (uint32_t)SH::B_BYTES;
+#pragma unroll
+                        for (int u = 0; u < SH::GS; ++u) {
+                            const int sl = g * SH::GS + u;
+                            if (sl >= SH::SLICES) break;
+                            const int ks = SH::slice_k(sl);
+                            const uint64_t ad = umma_desc(a0 + (uint32_t)(u * SH::A_SLICE), (uint32_t)ks * 16u);
+                            const uint64_t bd = umma_desc(b0 + (uint32_t)(NMAX * 2 * kKS * sl), (uint32_t)ks * 16u);
+#pragma unroll
+                            for (int kk = 0; kk < ks / 16; ++kk) {
+                                const uint32_t accum = (sl > 0 || kk > 0) ? 1u : 0u;
+                                asm volatile(
+                                    "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dt),
+                                    "l"(ad + 16u * kk), "l"(bd + 16u * kk), "r"(idesc), "r"(accum));
+                            }
                         }
                         issued = true;
                         umma_commit(&S.a_empty[a_i]);  // the stage is free once these MMAs are done
@@ -574,150 +621,146 @@ __global__ void __launch_bounds__(tc_threads(KP), 1) k_join_tc(JoinParams P, TcP
                 }
             }
         }
-    } else {
-        // ------------------------------------------------------------ epilogue
-        const int ew = warp - 3;
-        const int quarter = warp & 3;  // TMEM lanes 32 quarter .. + 31
-        const int part = ew >> 2;      // 32-column chunks part, part + EPI / 4, ...
-        const int row = quarter * 32 + lane;
+    } else if (warp == 3) {
+        // ------------------------------------------------------------ rows
+        // Four rows a lane: position, flag and thresholds of the next tile are
+        // fetched while the current one's are handed over, so that an epilogue
+        // warp reads 16 bytes a row and nothing else.
         const float* __restrict__ TO = static_cast<const float*>(P.thr_out);
         const float* __restrict__ TI = static_cast<const float*>(P.thr_in);
-        TcRecords rec{0, 0};
         uint32_t it_i = 0, it_ph = 0, m_i = 0, m_ph = 0, acc = 0, acc_ph = 0;
+        // (the loaded thresholds are first touched a tile later)
+        int32_t np[4], nfl[4];  // position, flag (-1: no candidate)
+        float nto[4], nti[4];
+        auto fetch = [&]() -> bool {
+            if (!bar_wait_warp(&S.meta_full[m_i], m_ph, abort)) return false;
+            const TcMeta& M = S.meta[m_i];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int row = 32 * u + lane;
+                const int4 g = M.g[row >> 3];
+                np[u] = g.x + (row & 7);
+                const bool valid = g.x >= 0 && np[u] >= g.y && np[u] < g.z &&
+                                   SJ_BOUND(P, np[u] < P.n_points, 31);
+                nfl[u] = valid ? g.w : -1;
+                const int32_t pl = valid ? np[u] : 0;
+                nto[u] = TO[pl];
+                nti[u] = TI[pl];
+            }
+            __syncwarp();
+            if (lane == 0) bar_arrive(&S.meta_empty[m_i]);
+            if (++m_i == kMetaDepth) m_i = 0, m_ph ^= 1u;
+            return true;
+        };
+        bool bail = false;
+        while (!bail) {
+            if (!bar_wait_warp(&S.item_full[it_i], it_ph, abort)) break;
+            const long long it = S.items[it_i].it;
+            const int ntiles = S.items[it_i].ntiles;
+            __syncwarp();
+            if (lane == 0) bar_arrive(&S.item_empty[it_i]);
+            if (it < 0) break;
+            if (++it_i == 2) it_i = 0, it_ph ^= 1u;
+            if (ntiles > 0 && !fetch()) break;
+            for (int t = 0; t < ntiles; ++t) {
+                int4 now[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    // (negated, never -0: the sign of a round-to-nearest sum
+                    // a + nto is that of the exact a - threshold)
+                    now[u] = make_int4(np[u], nfl[u], nfl[u] >= 0 ? __float_as_int(__fsub_rn(0.f, nto[u])) : (int)0xFF800000u,
+                                       nfl[u] >= 0 ? __float_as_int(__fsub_rn(0.f, nti[u])) : (int)0xFF800000u);
+                if ((t + 1 < ntiles && !fetch()) || !bar_wait_warp(&S.acc_empty[acc], acc_ph ^ 1u, abort)) {
+                    bail = true;
+                    break;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) S.rows[acc][32 * u + lane] = now[u];
+                __syncwarp();
+                if (lane == 0) bar_arrive(&S.acc_full[acc]);
+                if (++acc == 2) acc = 0, acc_ph ^= 1u;
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ epilogue
+        const int ew = warp - 4;
+        const int quarter = warp & 3;  // TMEM lanes 32 quarter .. + 31
+        const int part = ew >> 2;      // 32-column chunks part, part + EPI / 4, ...
+        constexpr int CSTEP = 32 * (SM::EPI / 4);
+        TcRecords rec{0, 0};
+        uint32_t it_i = 0, it_ph = 0, acc = 0, acc_ph = 0;
         for (;;) {
             if (!bar_wait_warp(&S.item_full[it_i], it_ph, abort)) break;
             const TcItem X = S.items[it_i];
             if (X.it < 0) break;
             bool fail = false;
-            // this thread's candidate row, read one tile ahead so its
-            // threshold loads overlap the previous tile
-            int32_t p = 0;
-            bool valid = false;
-            int fl = 0;
-            float to = INFINITY, ti = INFINITY;
-            auto read_meta = [&]() -> bool {
-                if (!bar_wait_warp(&S.meta_full[m_i], m_ph, abort)) return false;
-                const TcMeta& M = S.meta[m_i];
-                const int4 g = M.g[row >> 3];
-                p = g.x + (row & 7);
-                if (g.x >= 0 && !SJ_BOUND(P, p < P.n_points + kTcPadRows, 31)) p = 0;
-                valid = g.x >= 0 && p >= g.y && p < g.z;
-                fl = g.w;
-                __syncwarp();
-                if (lane == 0) bar_arrive(&S.meta_empty[m_i]);
-                if (++m_i == kMetaDepth) m_i = 0, m_ph ^= 1u;
-                // unconditional loads from an in-bounds row (selecting the
-                // loaded values here would wait for them; every use below
-                // is guarded by `valid`), so their latency overlaps the
-                // current tile's chunks
-                const int32_t pl = valid ? p : 0;
-                to = TO[pl];
-                ti = TI[pl];
-                return true;
-            };
-            if (X.ntiles > 0 && !read_meta()) fail = true;
-            const int cq0 = X.q0 - X.qa, cq1 = X.q1 - X.qa;  // the item's query columns
-            for (int t = 0; t < X.ntiles && !fail; ++t) {
-                const int32_t cp = p;
-                const bool cvalid = valid;
-                const int cfl = fl;
-                const float cto = to;
-                // negated thresholds, never -0: the sign of a round-to-nearest
-                // sum a + nto is that of the exact a - cto
-                const float nto = __fsub_rn(0.f, to), nti = __fsub_rn(0.f, ti);
-                // this row's valid query columns: the item's, and in a self-cell
-                // triangle those at or below the candidate (one unsigned compare)
-                const int col_lo = cq0;
-                const int col_hi = cfl == 2 ? min(cq1 - 1, cp - X.qa) : cq1 - 1;
-                const bool has_cols = col_hi >= col_lo;
-                const uint32_t col_span = has_cols ? (uint32_t)(col_hi - col_lo) : 0u;
+            for (int t = 0; t < X.ntiles; ++t) {
                 if (!bar_wait_warp(&S.acc_full[acc], acc_ph, abort)) {
                     fail = true;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;");
+                // this thread's candidate row
+                const int4 row = S.rows[acc][quarter * 32 + lane];
+                const int32_t cp = row.x;
+                const float nto = __int_as_float(row.z), nti = __int_as_float(row.w);
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + acc * NMAX;
-                constexpr int CSTEP = 32 * (SM::EPI / 4), UN = tc_chunks(KP);
-                // UN chunks at a time, their loads and the next tile's metadata
-                // in flight together; the accumulator is released as soon as
-                // this warp's last columns are in registers, before any of
-                // them is looked at
-                for (int c0 = 32 * part; c0 < X.ncol || c0 == 32 * part; c0 += UN * CSTEP) {
-                    // (whole chunks, no branches around the loads: columns past
-                    // the accumulated ones hold an earlier tile's and are left
-                    // out below)
-                    bool live[UN];
-                    uint32_t v[UN][32];
-#pragma unroll
-                    for (int u = 0; u < UN; ++u) {
-                        live[u] = c0 + u * CSTEP < X.ncol;
-                        tmem_ld32(taddr + (uint32_t)(live[u] ? c0 + u * CSTEP : 32 * part), v[u]);
-                    }
-                    if (c0 == 32 * part && t + 1 < X.ntiles && !read_meta()) fail = true;
+                // the accumulator is released as soon as this warp's last
+                // columns are in registers, before they are looked at
+                for (int c0 = 32 * part; c0 < X.ncol || c0 == 32 * part; c0 += CSTEP) {
+                    // (whole chunks, no branch around the load: columns past the
+                    // accumulated ones hold an earlier tile's and are left out below)
+                    uint32_t v[32];
+                    tmem_ld32(taddr + (uint32_t)c0, v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (X.ncol - c0 <= UN * CSTEP) {  // (this warp's last chunks)
+                    if (X.ncol - c0 <= CSTEP) {  // (this warp's last chunk)
                         asm volatile("tcgen05.fence::before_thread_sync;");
                         __syncwarp();
                         if (lane == 0) bar_arrive(&S.acc_empty[acc]);
+                        if (X.ncol <= c0) break;
                     }
-                    if (DBG && cvalid && has_cols) {  // the filter dump (test aid)
-                        // (constant indices: v stays in registers)
+                    // maxima of 8-column groups, then of all 32 (three-input max)
+                    const float* f = reinterpret_cast<const float*>(v);
+                    float m8[4];
 #pragma unroll
-                        for (int u = 0; u < UN; ++u)
+                    for (int g8 = 0; g8 < 4; ++g8)
+                        m8[g8] = max3f(max3f(f[8 * g8], f[8 * g8 + 1], f[8 * g8 + 2]),
+                                       max3f(f[8 * g8 + 3], f[8 * g8 + 4], f[8 * g8 + 5]),
+                                       fmaxf(f[8 * g8 + 6], f[8 * g8 + 7]));
+                    if (X.ncol - c0 < 32) m8[2] = m8[3] = -INFINITY;  // (a 16-column tail)
+                    const float top = max3f(m8[0], m8[1], fmaxf(m8[2], m8[3]));
+                    if (!DBG && !__any_sync(0xffffffffu, __fadd_rn(top, nto) >= 0.f)) continue;
+                    // this row's columns: the item's, and in a self-cell triangle
+                    // those at or below the candidate
+                    const int lo = max(X.q0 - X.qa - c0, 0);
+                    const int hi = min((row.y == 2 ? min(X.q1 - 1, cp) : X.q1 - 1) - X.qa - c0, 31);
+                    const uint32_t cols = lo <= hi && row.z != (int)0xFF800000u
+                                              ? (0xFFFFFFFFu << lo) & (0xFFFFFFFFu >> (31 - hi)) : 0u;
+                    if (DBG) {  // the filter dump (test aid; constant indices: v stays in registers)
 #pragma unroll
-                            for (int k = 0; k < 32; ++k) {
-                                const int col = c0 + u * CSTEP + k;
-                                if (col < X.ncol && (uint32_t)(col - col_lo) <= col_span)
-                                    dbg_record(P, X.qa + col, cp, __uint_as_float(v[u][k]));
-                            }
+                        for (int k = 0; k < 32; ++k)
+                            if (cols >> k & 1u) dbg_record(P, X.qa + c0 + k, cp, f[k]);
                     }
-                    // maxima of 8-column groups, then of all 32 (three-input
-                    // max), of all chunks before one is acted on
-                    float m8[UN][4];
-                    bool any[UN];
+                    // bit k: column c0 + k is maybe in / certainly in
+                    uint32_t mo = 0u, mi = 0u;
 #pragma unroll
-                    for (int u = 0; u < UN; ++u) {
-                        const float* f = reinterpret_cast<const float*>(v[u]);
+                    for (int g8 = 0; g8 < 4; ++g8) {
+                        if (!__any_sync(0xffffffffu, __fadd_rn(m8[g8], nto) >= 0.f)) continue;
+                        // sign of a - threshold: a miss
+                        uint32_t no = 0u, ni = 0u;
 #pragma unroll
-                        for (int g8 = 0; g8 < 4; ++g8)
-                            m8[u][g8] = max3f(max3f(f[8 * g8], f[8 * g8 + 1], f[8 * g8 + 2]),
-                                              max3f(f[8 * g8 + 3], f[8 * g8 + 4], f[8 * g8 + 5]),
-                                              fmaxf(f[8 * g8 + 6], f[8 * g8 + 7]));
-                        if (X.ncol - (c0 + u * CSTEP) < 32) m8[u][2] = m8[u][3] = -INFINITY;  // (a 16-column tail)
-                    }
-#pragma unroll
-                    for (int u = 0; u < UN; ++u)
-                        any[u] = __any_sync(0xffffffffu, live[u] && cvalid &&
-                                                          max3f(m8[u][0], m8[u][1], fmaxf(m8[u][2], m8[u][3])) >= cto);
-#pragma unroll
-                    for (int u = 0; u < UN; ++u) {
-                        const int cu = c0 + u * CSTEP;
-                        if (!any[u]) continue;
-                        const float* f = reinterpret_cast<const float*>(v[u]);
-                        // bit k: column cu + k is maybe in / certainly in
-                        uint32_t mo = 0u, mi = 0u;
-#pragma unroll
-                        for (int g8 = 0; g8 < 4; ++g8) {
-                            if (!__any_sync(0xffffffffu, cvalid && m8[u][g8] >= cto)) continue;
-                            // sign of a - threshold (see nto): a miss
-                            uint32_t no = 0u, ni = 0u;
-#pragma unroll
-                            for (int k = 6; k >= 0; k -= 2) {
-                                const float2 a = make_float2(f[8 * g8 + k], f[8 * g8 + k + 1]);
-                                const float2 o = __fadd2_rn(a, make_float2(nto, nto));
-                                const float2 n = __fadd2_rn(a, make_float2(nti, nti));
-                                no = push_sign(push_sign(no, o.y), o.x);
-                                ni = push_sign(push_sign(ni, n.y), n.x);
-                            }
-                            mo |= (~no & 0xFFu) << (8 * g8);
-                            mi |= (~ni & 0xFFu) << (8 * g8);
+                        for (int k = 6; k >= 0; k -= 2) {
+                            const float2 a = make_float2(f[8 * g8 + k], f[8 * g8 + k + 1]);
+                            const float2 o = __fadd2_rn(a, make_float2(nto, nto));
+                            const float2 n = __fadd2_rn(a, make_float2(nti, nti));
+                            no = push_sign(push_sign(no, o.y), o.x);
+                            ni = push_sign(push_sign(ni, n.y), n.x);
                         }
-                        // this row's columns (the item's, the triangle's)
-                        const int lo = max(col_lo - cu, 0), hi = min(col_hi - cu, 31);
-                        mo &= cvalid && lo <= hi ? (0xFFFFFFFFu << lo) & (0xFFFFFFFFu >> (31 - hi)) : 0u;
-                        tc_record(rec, P, lane, make_int4((int)mo, (int)mi, X.qa + cu,
-                                                          (int)((uint32_t)cp | (cfl ? kMirrorBit : 0u))));
+                        mo |= (~no & 0xFFu) << (8 * g8);
+                        mi |= (~ni & 0xFFu) << (8 * g8);
                     }
+                    tc_record(rec, P, lane, make_int4((int)(mo & cols), (int)mi, X.qa + c0,
+                                                      (int)((uint32_t)cp | (row.y ? kMirrorBit : 0u))));
                 }
                 if (++acc == 2) acc = 0, acc_ph ^= 1u;
             }
@@ -789,7 +832,7 @@ static int launch_kp(Index* ix, const JoinParams& p, const TcParams& t) {
     }
     SJ_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    constexpr int threads = tc_threads(KP);
+    constexpr int threads = kTcThreads;
     SJ_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     if (per_sm < 1) {
         set_error("tensor-core tile does not fit on an SM (K = %d)", KP);
