@@ -109,9 +109,9 @@ __global__ void k_knn_bucket(const int2* __restrict__ pairs, const double* __res
 // as an integer, and (distance bits, index) compare as one 96-bit integer: a
 // borrow chain of four 32-bit subtractions, no FP64 instruction (that pipe
 // runs at 1/64 of the integer rate here) and no case for equal distances.  A
-// bucket that fits the list, the usual case, is ranked once; a longer one is
-// cut back to its k smallest whenever the list is nearly full, and from then
-// on only entries below the k-th of those enter.  k rounds of a warp-wide
+// bucket that fits the list is ranked once; a longer one is cut back to its k
+// smallest whenever the list holds 2 k entries (at least 64), and from then on
+// only entries below the k-th of those enter: ranking m entries costs m^2.  k rounds of a warp-wide
 // minimum over the whole bucket, the earlier form, took a pass over the
 // bucket and ten shuffles per neighbour; it remains for k above kKnnCut with
 // longer buckets, which the list cannot hold.  Bound by instruction issue
@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(32 * kKnnWarps) k_knn_select(int64_t n, int k,
     const int found = (int)min(b - a, (uint32_t)k);
     if (b - a <= (uint32_t)kKnnList || k <= kKnnCut) {
         int4* list = s_list[threadIdx.x >> 5];
+        const int full = min(kKnnList - 31, max(64, 2 * k));  // cut back from this many on
         int m = 0;
         KnnKey bar{0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};  // the k-th smallest so far
         for (uint32_t s0 = a; s0 < b; s0 += 32) {
@@ -217,13 +218,16 @@ __global__ void __launch_bounds__(32 * kKnnWarps) k_knn_select(int64_t n, int k,
             if (in) list[m + __popc(w & ((1u << lane) - 1u))] = e;
             m += __popc(w);
             __syncwarp();
-            if (s0 == a && k <= kKnnEarly && b - a > 32u) {
-                knn_cut<1>(list, m, k, lane);
-                m = k;
-                bar = knn_key(list[k - 1]);
-            } else if (m > kKnnList - 32 && b - s0 > 32u && b - a > (uint32_t)kKnnList) {
-                // (a list this full holds more than k entries)
-                knn_cut<kKnnList / 32>(list, m, k, lane);
+            // (a list this full holds more than k entries, and room for 32)
+            if (b - s0 > 32u && (m >= full || (s0 == a && k <= kKnnEarly))) {
+                if (m <= 32)
+                    knn_cut<1>(list, m, k, lane);
+                else if (m <= 64)
+                    knn_cut<2>(list, m, k, lane);
+                else if (m <= 128)
+                    knn_cut<4>(list, m, k, lane);
+                else
+                    knn_cut<kKnnList / 32>(list, m, k, lane);
                 m = k;
                 bar = knn_key(list[k - 1]);
             }
