@@ -1897,6 +1897,7 @@ int build_index(Index* ix, const double* pts) {
         ix->n_items = (int64_t)(got.last_off & 0xFFFFFFFFull);
         ix->n_candidates =
             de.symmetric ? (int64_t)(2 * got.t.n_evaluated - got.t.sum_sq) : (int64_t)got.t.n_evaluated;
+        ix->sum_sq = (int64_t)got.t.sum_sq;
         ix->n_evaluated = (int64_t)(got.t.n_evaluated - (uses_triangle(ix) ? got.t.tri_skip : 0ull));
         if ((int64_t)(got.last_off >> 32) != n || (run_off && ix->n_runs > runs_cap) || ix->n_items > items_cap) {
             set_error("internal: dense index sizes inconsistent (%lld points, %lld runs, %lld items)",
@@ -1948,6 +1949,7 @@ int build_index(Index* ix, const double* pts) {
     ix->n_runs = (int64_t)tot.n_runs;
     ix->n_items = (int64_t)tot.n_items;
     ix->n_candidates = ep.symmetric ? (int64_t)(2 * tot.n_evaluated - tot.sum_sq) : (int64_t)tot.n_evaluated;
+    ix->sum_sq = (int64_t)tot.sum_sq;
     // the CUDA-core kernels evaluate only the triangle of each self cell
     ix->n_evaluated = (int64_t)(tot.n_evaluated - (uses_triangle(ix) ? tot.tri_skip : 0ull));
     if (tot.n_runs >= 0xFFFFFFFFull || tot.n_items >= 0x7FFFFFFFull) {

@@ -134,6 +134,7 @@ struct Index {
     Run* runs = nullptr;
     Item* items = nullptr;
     int64_t n_cells = 0, n_runs = 0, n_items = 0, n_candidates = 0, n_evaluated = 0;
+    int64_t sum_sq = 0;                 // sum over cells of their points squared
     double filter_band_rel = 0;  // predicted certified band (relative to eps^2)
     double bound_c1 = 0, bound_p = 0;  // certified bound E = c1 (P + pc) of the filter
     double kscale = 1.0;        // kernel coordinates = (x - centre) * kscale (a power of two)
@@ -310,8 +311,9 @@ constexpr int tc_qmax(int kp) { return tc_nmax(kp) - 8; }
 // groups and query tiles past the end read zeros.
 constexpr int kTcPadRows = 256;
 // Number of counters of a join (item queue, result cursor, rechecked,
-// recheck-queue fill, error flag, spare).
-constexpr int kCounters = 8;
+// recheck-queue fill, error flag, dump records, pruned, bounds check; queue and
+// length of the list of items that the sparse FP32 filter leaves).
+constexpr int kCounters = 10;
 int launch_join_dmma(Index* ix, const JoinOut& out, int emit_dist);
 
 // Queries per work item of an index: the caller's queries_per_item when set

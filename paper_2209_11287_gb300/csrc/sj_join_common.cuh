@@ -56,6 +56,10 @@ struct JoinParams {
     // pair evaluations this removes
     float prune_r2;
     float refine_out, refine_in;  // (Index: the same names; batched: per instance)
+    // FP32 filters, sparse indexes: work items that k_join_f32r leaves to
+    // k_join_f32s (counters[9] of them, taken through counters[8]); null: all
+    // items, through counters[0]
+    int32_t* big_items;
 };
 
 // Records one evaluated pair for the filter dump.
@@ -70,8 +74,11 @@ __device__ __forceinline__ void dbg_record_pruned(const JoinParams& P, int32_t q
     if (k < P.dbg_cap) P.dbg[k] = make_int4(qs, cs, 0, 1);
 }
 
-// The FP32 filter for sparse indexes (sj_join_f32r.cu).
-bool f32r_preferred(const Index* ix, const JoinParams& p);
+// The FP32 filter for sparse indexes (sj_join_f32r.cu): whether a join takes it
+// for no work item, for all, or for those of few queries (the others listed in
+// p.big_items), and its launch.
+enum class SparseUse { none, all, few_queries };
+SparseUse f32r_use(const Index* ix, const JoinParams& p);
 int launch_join_f32r(Index* ix, const JoinParams& p);
 
 JoinParams make_join_params(Index* ix, const JoinOut& out, int emit_dist);

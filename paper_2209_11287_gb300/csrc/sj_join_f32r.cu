@@ -24,6 +24,7 @@ namespace sj {
 namespace {
 
 constexpr int kF32rItems = 8;     // items a warp takes at a time
+constexpr int kF32rQ = 3;         // most queries of an item dealt with here when there is a list for the others
 constexpr int kF32rRuns = 256;    // runs of a group of them (an item has at most kMaxRuns)
 constexpr int kF32rStage = 256;
 constexpr int kF32rWarps = 4;
@@ -63,6 +64,19 @@ __global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P) {
         if (lane < kF32rItems && first + lane < P.n_items) I = P.items[first + lane];
         if (!SJ_BOUND(P, I.q0 >= 0 && I.q1 <= P.n_points && I.r1 - I.r0 <= kF32rRuns, 51)) I = Item{0, 0, 0, 0};
         const int have = (int)min((long long)kF32rItems, P.n_items - first);
+        if (P.big_items) {  // items of many queries are left to k_join_f32s
+            const bool big = I.q1 - I.q0 > kF32rQ;
+            const unsigned m = __ballot_sync(0xffffffffu, big);
+            if (m) {
+                unsigned long long at = 0;
+                if (lane == 0) at = atomicAdd(&P.counters[9], (unsigned long long)__popc(m));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (big) {
+                    P.big_items[at + __popc(m & ((1u << lane) - 1u))] = (int32_t)(first + lane);
+                    I = Item{0, 0, 0, 0};
+                }
+            }
+        }
         int upto = I.r1 - I.r0;  // inclusive prefix of the items' runs
 #pragma unroll
         for (int o = 1; o < kF32rItems; o <<= 1) {
@@ -205,19 +219,26 @@ int launch_f32r_d(Index* ix, const JoinParams& p) {
 
 }  // namespace
 
-// Taken for single joins when cells are sparse: fewer than 2.5 queries an item
-// (1.9 for padded d = 8, whose candidates cost more to load) and, against a few
-// crowded cells among many single ones, fewer than 160 (300) evaluations an
-// item.  Both kernels, us, by queries an item: uniform 4-D 1.1 754 / 155, 1.4
-// 667 / 274, 2.0 540 / 352, 3.2 419 / 475; 3-D 1.6 283 / 88, 3.9 156 / 151; 2-D
-// 1.8 375 / 164, 2.8 286 / 210, 5.1 195 / 279; 5-D 1.8 323 / 245, 3.8 266 / 500;
-// 6-D 1.2 336 / 189, 1.8 348 / 382; clusters over noise, 3-D 1.6 464 / 333, 2.7
-// 387 / 927.  (Batched joins and the filter's recording mode keep k_join_f32s.)
-bool f32r_preferred(const Index* ix, const JoinParams& p) {
-    if (p.batch || p.dbg || ix->n_cells <= 0) return false;
-    const double items = (double)ix->n_cells + (double)ix->n / kQMax;
-    return ix->dp <= 4 ? (double)ix->n < 2.5 * items && (double)ix->n_evaluated < 160.0 * items
-                       : (double)ix->n < 1.9 * items && (double)ix->n_evaluated < 300.0 * items;
+// Taken for single joins whose cells are sparse.  Evenly filled cells (a point's
+// own cell holds at most 1.6 times the mean cell): for all items below 2.5
+// queries an item (1.9 for padded d = 8, whose candidates cost more to load) and
+// 160 (300) evaluations an item.  Both kernels, us, by queries an item: uniform
+// 4-D 1.1 754 / 155, 1.4 667 / 274, 2.0 540 / 352, 3.2 419 / 475; 3-D 1.6 283 /
+// 88, 3.9 156 / 151; 2-D 1.8 375 / 164, 2.8 286 / 210, 5.1 195 / 279; 5-D 1.8
+// 323 / 245, 3.8 266 / 500; 6-D 1.2 336 / 189, 1.8 348 / 382.  Crowded and single
+// cells side by side: for the items of up to 3 queries, below 3.2 queries an item
+// as n / (cells + n / 16) counts them (clusters over noise, k_join_f32s alone / k_join_f32r alone / shared: 3-D 1.6
+// 467 / 333 / 315, 2.7 389 / 927 / 346, 4-D 2.3 596 / - / 485, 2-D 3.2 337 / 488 /
+// 293, 4.7 154 / - / 166; at 2 and 4 queries 347 and 362 for the 3-D 2.7; shared
+// on even cells it costs the second launch: uniform 4-D 1.4 305).  (Batched joins
+// and the filter's recording mode keep k_join_f32s.)
+SparseUse f32r_use(const Index* ix, const JoinParams& p) {
+    if (p.batch || p.dbg || ix->n_cells <= 0) return SparseUse::none;
+    const double n = (double)ix->n, cells = (double)ix->n_cells, items = cells + n / kQMax;
+    if ((double)ix->sum_sq / n > 1.6 * n / cells) return n < 3.2 * items ? SparseUse::few_queries : SparseUse::none;
+    const bool small = ix->dp <= 4;
+    return n < (small ? 2.5 : 1.9) * items && (double)ix->n_evaluated < (small ? 160.0 : 300.0) * items ? SparseUse::all
+                                                                                               : SparseUse::none;
 }
 
 int launch_join_f32r(Index* ix, const JoinParams& p) {

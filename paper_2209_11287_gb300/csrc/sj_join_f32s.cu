@@ -458,7 +458,9 @@ constexpr int f32s_min_blocks() {
     return DP == 2 ? SJ_F32S_MIN_BLOCKS_D2 : DP == 4 ? SJ_F32S_MIN_BLOCKS_D4 : SJ_F32S_MIN_BLOCKS_D8;
 }
 
-template <int DP, int RUNS, bool DBG>
+// LISTED: the items are those that k_join_f32r listed (an instantiation of its
+// own: the indirection costs the kernel for all items 2%).
+template <int DP, int RUNS, bool DBG, bool LISTED>
 __global__ void __launch_bounds__(kF32sWarps * 32, f32s_min_blocks<DP>()) k_join_f32s(JoinParams P) {
     constexpr int TC = f32s_tc<DP>();
     constexpr uint32_t SLOTS = 32u * TC;
@@ -476,13 +478,16 @@ __global__ void __launch_bounds__(kF32sWarps * 32, f32s_min_blocks<DP>()) k_join
         W.smir = 0;
     }
 
+    constexpr int QUEUE = LISTED ? 8 : 0;
+    long long listed = 0;
+    if constexpr (LISTED) listed = (long long)P.counters[9];
     long long next = 0;
-    if (lane == 0) next = (long long)atomicAdd(&P.counters[0], 1ull);
+    if (lane == 0) next = (long long)atomicAdd(&P.counters[QUEUE], 1ull);
     next = __shfl_sync(0xffffffffu, next, 0);
     for (;;) {
-        const long long it = next;
-        if (it >= P.n_items) break;
-        if (lane == 0) next = (long long)atomicAdd(&P.counters[0], 1ull);  // used next iteration
+        if (next >= (LISTED ? listed : P.n_items)) break;
+        const long long it = LISTED ? (long long)P.big_items[next] : next;
+        if (lane == 0) next = (long long)atomicAdd(&P.counters[QUEUE], 1ull);  // used next iteration
         next = __shfl_sync(0xffffffffu, next, 0);
         const Item I = P.items[it];
         const int Q = I.q1 - I.q0;
@@ -572,9 +577,9 @@ __global__ void __launch_bounds__(kF32sWarps * 32, f32s_min_blocks<DP>()) k_join
     if (lane == 0 && W.pruned) atomicAdd(&P.counters[6], W.pruned);
 }
 
-template <int DP, int RUNS, bool DBG>
+template <int DP, int RUNS, bool DBG, bool LISTED>
 static int launch_f32s_dr(Index* ix, const JoinParams& p) {
-    auto kern = k_join_f32s<DP, RUNS, DBG>;
+    auto kern = k_join_f32s<DP, RUNS, DBG, LISTED>;
     static std::atomic<int> cached{0};  // resident CTAs per SM (a property of the kernel)
     int per_sm = cached.load(std::memory_order_relaxed);
     if (per_sm == 0) {
@@ -593,8 +598,10 @@ static int launch_f32s_dr(Index* ix, const JoinParams& p) {
 
 template <int DP>
 static int launch_f32s_d(Index* ix, const JoinParams& p) {
-    if (p.dbg) return launch_f32s_dr<DP, kMaxRuns, true>(ix, p);  // the filter dump (test aid)
-    return ix->m <= 4 ? launch_f32s_dr<DP, 28, false>(ix, p) : launch_f32s_dr<DP, kMaxRuns, false>(ix, p);
+    if (p.dbg) return launch_f32s_dr<DP, kMaxRuns, true, false>(ix, p);  // the filter dump (test aid)
+    if (p.big_items)
+        return ix->m <= 4 ? launch_f32s_dr<DP, 28, false, true>(ix, p) : launch_f32s_dr<DP, kMaxRuns, false, true>(ix, p);
+    return ix->m <= 4 ? launch_f32s_dr<DP, 28, false, false>(ix, p) : launch_f32s_dr<DP, kMaxRuns, false, false>(ix, p);
 }
 
 bool f32s_supported(const Index* ix, int emit_dist) {
@@ -602,8 +609,12 @@ bool f32s_supported(const Index* ix, int emit_dist) {
 }
 
 int launch_join_f32s(Index* ix, const JoinOut& out) {
-    const JoinParams p = make_join_params(ix, out, 0);
-    if (f32r_preferred(ix, p)) return launch_join_f32r(ix, p);
+    JoinParams p = make_join_params(ix, out, 0);
+    Scratch tmp(ix->stream);  // (released after the launches that use it, stream-ordered)
+    const SparseUse sparse = f32r_use(ix, p);
+    if (sparse == SparseUse::few_queries) SJ_TRY(tmp.alloc(&p.big_items, (size_t)ix->n_items));
+    if (sparse != SparseUse::none) SJ_TRY(launch_join_f32r(ix, p));
+    if (sparse == SparseUse::all) return SJ_OK;
     switch (ix->dp) {
         case 2: return launch_f32s_d<2>(ix, p);
         case 4: return launch_f32s_d<4>(ix, p);

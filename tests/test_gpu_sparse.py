@@ -1,4 +1,4 @@
-"""The FP32 filter for sparse cells (k_join_f32r): groups of items whose runs
+"""The FP32 filter for sparse cells (k_join_f32r), alone and beside k_join_f32s: groups of items whose runs
 fill the warp's list (27, 81 and 243 runs an item), items of one and of several
 queries, uncertain pairs and a recheck queue that overflows nowhere, ranges of
 items and rounds to the host, symmetric and not; the oracle's pair set, and the
@@ -19,13 +19,17 @@ def _set(kind, n, d, g):
         return g.random((n, d)), (0.35 / n) ** (1.0 / d)
     if kind == "lattice":  # many pairs at exactly eps (uncertain), few points a cell
         return g.integers(0, int(2 * n ** (1.0 / d)), size=(n, d)) / 8.0, 1.0 / 8.0
+    if kind == "crowded":  # a few crowded cells among single points: both kernels share the items
+        x = g.random((n, d))
+        x[: n // 3] = 0.5 + 0.02 * (g.random((n // 3, d)) - 0.5) + 0.25 * g.integers(0, 2, (n // 3, 1))
+        return x, (0.3 / n) ** (1.0 / d)
     x = g.random((n, d))  # near-duplicates of a few points among single ones
     x[: n // 8] = x[g.integers(n // 8, n // 6, n // 8)] + 1e-9 * g.standard_normal((n // 8, d))
     return x, (0.3 / n) ** (1.0 / d)
 
 
 @pytest.mark.parametrize("symmetric", [True, False])
-@pytest.mark.parametrize("kind", ["uniform", "lattice", "duplicates"])
+@pytest.mark.parametrize("kind", ["uniform", "lattice", "duplicates", "crowded"])
 @pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 6, 8])
 def test_sparse_cells(d, kind, symmetric):
     if not torch.cuda.is_available():
