@@ -24,6 +24,8 @@ namespace sj {
 namespace {
 
 constexpr int kResolveWarps = 4;
+constexpr int kResolveBlocks = 8;
+constexpr int kResolveRun = 16;  // blocks of 32 records that one warp takes in a row, at most
 
 // Squared distance of two kernel-coordinate rows, binary32.
 template <int DP>
@@ -49,8 +51,13 @@ __device__ __forceinline__ float refine_sq(const float* __restrict__ a, const fl
     return s;
 }
 
+// Bound by the latency of its gathers (positions to ids and rows, cursor and
+// page of a flush), so a pair's first loads do not wait for one another
+// (500,000 x 16-D mixture, build, filter and this kernel: the ids loaded after
+// the decision 2.69 ms, before it 2.64).  8 CTAs an SM leave 64 registers a
+// thread; 10, 12 and 16 were slower (2.73, 2.81 ms and more, by the spills).
 template <int DP, bool EMIT>
-__global__ void __launch_bounds__(32 * kResolveWarps) k_resolve(JoinParams P) {
+__global__ void __launch_bounds__(32 * kResolveWarps, kResolveBlocks) k_resolve(JoinParams P) {
     __shared__ int2 s_stage[kResolveWarps][kStage];
     __shared__ double s_sdist[kResolveWarps][EMIT ? kStage : 1];
     // pairs waiting: (query position | certain << 31, candidate position | mirrored << 31)
@@ -61,6 +68,9 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_resolve(JoinParams P) {
     int2* list = s_list[wid];
     int waiting = 0;
     unsigned long long decided = 0;
+    const int32_t* __restrict__ inst_of = P.batch ? P.batch->inst_of_sorted : nullptr;
+    const int32_t* __restrict__ inst_gid = P.batch ? P.batch->inst_gid : nullptr;
+    const long long* __restrict__ inst_off = P.batch ? P.batch->inst_off : nullptr;
 
     // 32 pairs, one a lane
     auto deal = [&](bool live, int2 e) {
@@ -68,35 +78,30 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_resolve(JoinParams P) {
         live = live && SJ_BOUND(P, qs < P.n_points && cs < P.n_points, 41);
         const bool certain = !EMIT && e.x < 0;
         int nout = 0, gid = 0;
-        int32_t qid = 0, cid = 0, off = 0;
+        int32_t qid = 0, cid = 0;
         double dist = 0.0;
         if (live) {
-            float r_out = P.refine_out, r_in = P.refine_in;
-            double e2 = P.e2;
-            if (P.batch) {
-                const int li = P.batch->inst_of_sorted[qs];
-                const float2 r = P.batch->inst_refine[li];
-                r_out = r.x;
-                r_in = r.y;
-                e2 = P.batch->inst_e2[li];
-                gid = P.batch->inst_gid[li];
-                off = (int32_t)P.batch->inst_off[li];
-            }
+            qid = P.perm[qs];
+            cid = P.perm[cs];
+            const int li = inst_of ? inst_of[qs] : 0;
             bool in = certain;
             if (!certain) {
                 ++decided;
                 const float s32 = refine_sq<DP>(Y + (int64_t)qs * DP, Y + (int64_t)cs * DP);
-                in = s32 < r_in;
-                if (EMIT ? !(s32 > r_out) : !in && !(s32 > r_out)) {
+                const float2 r = inst_of ? P.batch->inst_refine[li] : make_float2(P.refine_out, P.refine_in);
+                in = s32 < r.y;
+                if (EMIT ? !(s32 > r.x) : !in && !(s32 > r.x)) {
                     const double s = direct_sq(P.xs + (int64_t)qs * DP, P.xs + (int64_t)cs * DP, P.d);
-                    in = s <= e2;
+                    in = s <= (inst_of ? P.batch->inst_e2[li] : P.e2);
                     if (EMIT && in) dist = sqrt(s);
                 }
             }
-            if (in) {
-                nout = e.y < 0 && cs != qs ? 2 : 1;
-                qid = P.perm[qs] - off;
-                cid = P.perm[cs] - off;
+            if (in) nout = e.y < 0 && cs != qs ? 2 : 1;
+            if (inst_of) {
+                gid = inst_gid[li];
+                const int32_t off = (int32_t)inst_off[li];
+                qid -= off;
+                cid -= off;
             }
         }
         if (P.batch) {
@@ -122,9 +127,35 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_resolve(JoinParams P) {
     const int4* __restrict__ records = reinterpret_cast<const int4*>(P.band);
     const unsigned long long taken = P.counters[3], room = P.band_cap >> 1;
     const unsigned long long count = taken < room ? taken : room;
-    const unsigned long long step = (unsigned long long)gridDim.x * kResolveWarps * 32;
-    for (unsigned long long b = ((unsigned long long)blockIdx.x * kResolveWarps + wid) * 32; b < count; b += step) {
+    // A warp takes up to kResolveRun blocks of 32 records that follow one
+    // another: in a batch they come from the same few instances, so the stage
+    // fills before the instance changes (blocks a grid apart changed it nearly
+    // every time: a flush, with its atomic on the instance's cursor, for 32
+    // records, and a warp of mixed leftovers written pair by pair).  Measured,
+    // 96 joins in one batch: blocks a grid apart 6.52 ms, runs of 4 6.22, 16
+    // 6.19, 64 6.17; one join of the 16-D mixture 2.64 / 2.67 / 2.67 / 2.77 ms,
+    // long runs leave warps idle.
+    const unsigned long long warps = (unsigned long long)gridDim.x * kResolveWarps, blocks = (count + 31) / 32;
+    const unsigned long long run = min((unsigned long long)kResolveRun, max(1ull, blocks / (2 * warps)));
+    int of_list = -1;  // batch: the instance of the waiting pairs
+    unsigned long long r = (unsigned long long)blockIdx.x * kResolveWarps + wid, k_run = 0;
+    for (; r * run + k_run < blocks; k_run + 1 < run ? ++k_run : (k_run = 0, r += warps)) {
+        const unsigned long long b = (r * run + k_run) * 32;
         const int4 e = b + lane < count ? records[b + lane] : make_int4(0, 0, 0, 0);
+        if (inst_of) {  // what waits of another instance goes first, so that a warp of pairs has one
+            const int cs = (int)((uint32_t)e.w & ~kMirrorBit);
+            const unsigned some = __ballot_sync(0xffffffffu, e.x != 0);
+            if (some == 0u) continue;
+            int li = e.x != 0 && SJ_BOUND(P, cs < P.n_points, 41) ? inst_of[cs] : 0;
+            li = __shfl_sync(0xffffffffu, li, __ffs(some) - 1);
+            if (waiting > 0 && li != of_list) {
+                __syncwarp();
+                deal(lane < waiting, list[lane < waiting ? lane : 0]);
+                __syncwarp();
+                waiting = 0;
+            }
+            of_list = li;
+        }
         uint32_t m = (uint32_t)e.x;
         for (;;) {  // a column of every record at a time into the list
             const unsigned w = __ballot_sync(0xffffffffu, m != 0u);
@@ -153,7 +184,7 @@ __global__ void __launch_bounds__(32 * kResolveWarps) k_resolve(JoinParams P) {
 
 template <int DP>
 int launch_resolve_dp(Index* ix, const JoinParams& p) {
-    const unsigned blocks = (unsigned)device_sm_count(ix->device) * 8;
+    const unsigned blocks = (unsigned)device_sm_count(ix->device) * kResolveBlocks;
     if (p.emit_dist)
         k_resolve<DP, true><<<blocks, 32 * kResolveWarps, 0, ix->stream>>>(p);
     else

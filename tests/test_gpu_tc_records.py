@@ -67,3 +67,16 @@ def test_batch_of_small_instances(emit):
         assert np.array_equal(key[order], ref)
         if emit:
             assert np.array_equal(dist[order], rd)
+
+
+def test_batch_of_many_records():
+    """Enough of them that a warp takes several blocks of records in a row,
+    over the edges of instances."""
+    g = np.random.Generator(np.random.PCG64(4))
+    xs = [g.random((int(m), 2)) for m in g.integers(100, 1800, 48)]
+    eps = [float(np.sqrt(120 / (np.pi * len(x)))) for x in xs]
+    out = binding.join_batch([torch.from_numpy(x).cuda() for x in xs], eps, kernel="filter_fp16x2",
+                             queries_per_item=1)
+    for x, e, (pairs, _, _) in zip(xs, eps, out):
+        ref, _ = oracle.join(x, e, with_dist=True)
+        assert np.array_equal(np.sort((pairs[:, 0].astype(np.int64) << 32) | pairs[:, 1]), ref)
