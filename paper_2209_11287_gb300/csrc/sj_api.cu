@@ -290,6 +290,21 @@ static int copy_pages(const T* const* pages, int n_pages, int64_t page_pairs, in
     return SJ_OK;
 }
 
+// The recheck queue of a join (queue_entries).  When memory is short, a
+// tensor-core filter makes do with the pairs' own share: the tile kernel deals
+// with the records past the queue.
+static int alloc_queue(int2** band, unsigned long long* cap, int kernel, unsigned long long ev, bool dist,
+                       cudaStream_t s) {
+    *cap = queue_entries(kernel, ev, dist);
+    int st = dev_alloc_t(band, (size_t)*cap, s);
+    const unsigned long long least = std::max<unsigned long long>(ev / (dist ? 8 : 64), 1ull << 20);
+    if (st == SJ_ERR_OOM && *cap > least) {
+        *cap = least;
+        st = dev_alloc_t(band, (size_t)least, s);
+    }
+    return st;
+}
+
 }  // namespace sj
 
 using namespace sj;
@@ -537,10 +552,11 @@ static int run_join(sj_index* ix, ResultImpl* ri, int64_t page_pairs, bool dist,
     // deferred-recheck queue: band pairs (and, with distances, every
     // maybe-in pair); pairs past its end are re-decided in place
     const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
-    const unsigned long long band_cap = queue_entries(ix->kernel, ev, dist);
     Scratch tmp(s);
     int2* band = nullptr;
-    SJ_TRY(tmp.alloc(&band, (size_t)band_cap));
+    unsigned long long band_cap = 0;
+    SJ_TRY(alloc_queue(&band, &band_cap, ix->kernel, ev, dist, s));
+    tmp.ptrs.push_back(band);
     JoinOut jo;
     jo.out_pairs = reinterpret_cast<int2*>(ri->block);
     jo.out_dist = ri->dblock;
@@ -619,7 +635,7 @@ int sj_self_join_to_host(sj_handle h, int32_t* host_pairs, int64_t host_capacity
     cudaStream_t s = ix->stream;
     const int64_t n_items = ix->n_items;
     const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
-    const unsigned long long band_cap = queue_entries(ix->kernel, ev, false);
+    unsigned long long band_cap = 0;
     int2* pool[2] = {nullptr, nullptr};
     int2* band = nullptr;
     cudaStream_t cs = nullptr;
@@ -627,7 +643,7 @@ int sj_self_join_to_host(sj_handle h, int32_t* host_pairs, int64_t host_capacity
     int st = SJ_OK;
     if ((st = dev_alloc_t(&pool[0], (size_t)device_pairs, s)) == SJ_OK &&
         (st = dev_alloc_t(&pool[1], (size_t)device_pairs, s)) == SJ_OK)
-        st = dev_alloc_t(&band, (size_t)band_cap, s);
+        st = alloc_queue(&band, &band_cap, ix->kernel, ev, false, s);
     if (st == SJ_OK) {
         cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
         for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
@@ -1337,8 +1353,8 @@ int join_batch_impl(const double* const* pts, const int64_t* n, const int32_t* d
             Index* ix = &g.ix;
             if (ix->n_items == 0) continue;
             const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
-            const unsigned long long band_cap = queue_entries(ix->kernel, ev, dist);
-            if ((st = dev_alloc_t(&bands[gi], (size_t)band_cap, s)) != SJ_OK) break;
+            unsigned long long band_cap = 0;
+            if ((st = alloc_queue(&bands[gi], &band_cap, ix->kernel, ev, dist, s)) != SJ_OK) break;
             jos[gi].band = bands[gi];
             jos[gi].band_cap = band_cap;
             jos[gi].batch = dbj + gi;
