@@ -111,14 +111,15 @@ __global__ void k_knn_bucket(const int2* __restrict__ pairs, const double* __res
 // runs at 1/64 of the integer rate here) and no case for equal distances.  A
 // bucket that fits the list is ranked once; a longer one is cut back to its k
 // smallest whenever the list holds 2 k entries (at least 64), and from then on
-// only entries below the k-th of those enter: ranking m entries costs m^2.  k rounds of a warp-wide
-// minimum over the whole bucket, the earlier form, took a pass over the
-// bucket and ten shuffles per neighbour; it remains for k above kKnnCut with
-// longer buckets, which the list cannot hold.  Bound by instruction issue
-// (four instructions per pair of entries and lane).  Measured, rounds / list:
-// 200,003 points, 47 neighbours, k = 16: 3424 / 150 us; 200,000 points, 57
-// neighbours, k = 8: 1798 / 149 us; 100,000 16-D points, 50 neighbours on
-// average, k = 32: 2943 / 299 us.
+// only entries below the k-th of those enter: ranking m entries costs m^2.  k
+// rounds of a warp-wide minimum over the whole bucket, the earlier form, took a
+// pass over the bucket and ten shuffles per neighbour; it remains for k above
+// kKnnCut with longer buckets, which the list cannot hold.  Bound by
+// instruction issue (four instructions per pair of entries and lane).
+// Measured, rounds / list: 200,003 points, 47 neighbours, k = 16: 3424 / 150
+// us; 200,000 points, 57 neighbours, k = 8: 1798 / 149 us; 100,000 16-D points,
+// 50 neighbours on average, k = 32: 2943 / 166 us (cut back at the full list
+// only: 299).
 constexpr int kKnnList = 256;            // list entries of a warp (4 KB)
 constexpr int kKnnCut = kKnnList - 64;   // largest k the list is cut back to
 // Up to this k the first 32 neighbours are cut back at once: the k-th of them
