@@ -14,6 +14,7 @@
 #include <algorithm>
 
 #include "sj_internal.cuh"
+#include "sj_knn_list.cuh"
 
 namespace sj {
 
@@ -120,7 +121,6 @@ __global__ void k_knn_bucket(const int2* __restrict__ pairs, const double* __res
 // us; 200,000 points, 57 neighbours, k = 8: 1798 / 149 us; 100,000 16-D points,
 // 50 neighbours on average, k = 32: 2943 / 166 us (cut back at the full list
 // only: 299).
-constexpr int kKnnList = 256;            // list entries of a warp (4 KB)
 constexpr int kKnnCut = kKnnList - 64;   // largest k the list is cut back to
 // Up to this k the first 32 neighbours are cut back at once: the k-th of them
 // keeps most of the rest out, and the final ranking is over about
@@ -128,69 +128,6 @@ constexpr int kKnnCut = kKnnList - 64;   // largest k the list is cut back to
 // us with; the two rankings cost more than the one from about 3/4 of 32 on).
 constexpr int kKnnEarly = 24;
 constexpr int kKnnWarps = 8;
-
-struct KnnKey {
-    uint32_t i, lo, hi;  // index, low and high half of the distance's bits
-};
-__device__ __forceinline__ KnnKey knn_key(int4 e) { return {(uint32_t)e.z, (uint32_t)e.x, (uint32_t)e.y}; }
-
-// r - 1 when a < b, else r.
-__device__ __forceinline__ int knn_minus_lt(int r, KnnKey a, KnnKey b) {
-    asm("{\n.reg .u32 t;\nsub.cc.u32 t, %1, %4;\nsubc.cc.u32 t, %2, %5;\nsubc.cc.u32 t, %3, %6;\n"
-        "subc.u32 %0, %0, 0;\n}"
-        : "+r"(r)
-        : "r"(a.i), "r"(a.lo), "r"(a.hi), "r"(b.i), "r"(b.lo), "r"(b.hi));
-    return r;
-}
-
-// The entries 32 u + lane (u < E) of a list of m <= 32 E entries and their
-// ranks (kKnnList past the end).
-template <int E>
-__device__ __forceinline__ void knn_rank(const int4* list, int m, int lane, int4 (&e)[E], int (&rank)[E]) {
-    KnnKey key[E];
-#pragma unroll
-    for (int u = 0; u < E; ++u) {
-        e[u] = list[min(32 * u + lane, m - 1)];
-        key[u] = knn_key(e[u]);
-        rank[u] = 0;
-    }
-#pragma unroll 4
-    for (int j = 0; j < m; ++j) {
-        const KnnKey o = knn_key(list[j]);
-#pragma unroll
-        for (int u = 0; u < E; ++u) rank[u] = knn_minus_lt(rank[u], o, key[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < E; ++u) rank[u] = 32 * u + lane < m ? -rank[u] : kKnnList;
-}
-
-// Cuts a list of m > k entries back to its k smallest, in order.
-template <int E>
-__device__ __forceinline__ void knn_cut(int4* list, int m, int k, int lane) {
-    int4 e[E];
-    int rank[E];
-    knn_rank<E>(list, m, lane, e, rank);
-    __syncwarp();
-#pragma unroll
-    for (int u = 0; u < E; ++u)
-        if (rank[u] < k) list[rank[u]] = e[u];
-    __syncwarp();
-}
-
-// Writes the min(m, k) smallest of the list as row i of the outputs.
-template <int E>
-__device__ __forceinline__ void knn_write(const int4* list, int m, int k, int64_t i, int lane, int32_t* idx_out,
-                                          double* dist_out) {
-    int4 e[E];
-    int rank[E];
-    knn_rank<E>(list, m, lane, e, rank);
-#pragma unroll
-    for (int u = 0; u < E; ++u)
-        if (rank[u] < k) {
-            idx_out[i * k + rank[u]] = e[u].z;
-            dist_out[i * k + rank[u]] = __hiloint2double(e[u].y, e[u].x);
-        }
-}
 
 __global__ void __launch_bounds__(32 * kKnnWarps) k_knn_select(int64_t n, int k, const uint32_t* __restrict__ off,
                                                                const KnnEntry* __restrict__ nb, int32_t* idx_out,
