@@ -277,9 +277,11 @@ int launch_recheck(Index* ix, const JoinOut& out, int emit_dist);
 int launch_resolve(Index* ix, const JoinOut& out, int emit_dist);
 // Entries (8 bytes) of the recheck queue of a join of `ev` evaluations.  A
 // tensor-core filter keeps its 16-byte records there, one per candidate and 32
-// query columns with a maybe-in pair: at most ev / 16 of them (records past
-// the queue are dealt with in the tile kernel), at most 2 GB above the pairs'
-// own share.
+// query columns with a maybe-in pair: room for ev / 16 of them, at most 2 GB or
+// the pairs' own share, which is a record of every 128 evaluations (16 with
+// distances).  More come of items of few queries (up to one per evaluation) and,
+// above 2^31 evaluations, of joins with a pair in most blocks of 32: the tile
+// kernel deals with the records past the queue.
 inline unsigned long long queue_entries(int kernel, unsigned long long ev, bool dist) {
     const unsigned long long small = ev / (dist ? 8 : 64), least = 1ull << 20;
     unsigned long long cap = small;
