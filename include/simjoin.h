@@ -570,11 +570,16 @@ SJ_API int sj_index_phase_ms(sj_handle h, double* device_ms, double* host_ms);
  * No counterpart in the paper.  sj_debug_fail_allocations(k): the library's
  * next k device allocations succeed and every later one fails with
  * SJ_ERR_OOM until the injection is switched off with a negative k
- * (process-wide, all threads).  sj_debug_live_allocations(): device blocks
+ * (process-wide, all threads).  sj_debug_fail_some_allocations(k, c): the next
+ * k succeed, the c after them fail, later ones succeed again (c = 0: off), as
+ * where a large block finds no room and a smaller one does; returns how many
+ * failures of the setting before were still due.
+ * sj_debug_live_allocations(): device blocks
  * the library holds at the moment (allocated and not yet released); a call
  * that fails must leave it where it was.
  */
 SJ_API void sj_debug_fail_allocations(int64_t after);
+SJ_API int64_t sj_debug_fail_some_allocations(int64_t after, int64_t count);
 SJ_API int64_t sj_debug_live_allocations(void);
 
 /* ---- status ------------------------------------------------------------ */

@@ -182,6 +182,8 @@ def load():
         lib.sj_index_perm.restype = ctypes.c_int
         lib.sj_debug_fail_allocations.argtypes = [_i64]
         lib.sj_debug_fail_allocations.restype = None
+        lib.sj_debug_fail_some_allocations.argtypes = [_i64, _i64]
+        lib.sj_debug_fail_some_allocations.restype = _i64
         lib.sj_debug_live_allocations.argtypes = []
         lib.sj_debug_live_allocations.restype = ctypes.c_int64
         lib.sj_index_item_work.argtypes = [_vp, _vp]
@@ -570,6 +572,13 @@ def sj_debug_fail_allocations(after: int) -> None:
     """Test aid: the next ``after`` device allocations succeed, later ones fail
     with SJ_ERR_OOM; a negative value switches the injection off."""
     load().sj_debug_fail_allocations(int(after))
+
+
+def sj_debug_fail_some_allocations(after: int, count: int) -> int:
+    """Test aid: the next ``after`` device allocations succeed, the ``count``
+    after them fail with SJ_ERR_OOM, later ones succeed (0: off).  Returns the
+    failures of the setting before that were still due."""
+    return load().sj_debug_fail_some_allocations(int(after), int(count))
 
 
 def sj_debug_live_allocations() -> int:

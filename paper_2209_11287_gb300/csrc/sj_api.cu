@@ -89,8 +89,10 @@ static int pool_for(int dev, cudaMemPool_t* out) {
 }
 
 // Test aid: allocations still allowed before injected failures start (-1:
-// no injection), and the device blocks currently held.
+// no injection), the same with a number of failures after which allocations
+// succeed again, and the device blocks currently held.
 static std::atomic<long long> g_fail_after{-1};
+static std::atomic<long long> g_fail_skip{0}, g_fail_some{0};
 static std::atomic<long long> g_live_blocks{0};
 
 void* host_staging(size_t bytes) {
@@ -119,9 +121,17 @@ void* host_staging(size_t bytes) {
 
 int dev_alloc(void** p, size_t bytes, cudaStream_t s) {
     *p = nullptr;
+    bool fail = false;
     if (g_fail_after.load(std::memory_order_relaxed) >= 0 &&
         g_fail_after.fetch_sub(1, std::memory_order_relaxed) <= 0) {
         g_fail_after.store(0, std::memory_order_relaxed);
+        fail = true;
+    }
+    if (g_fail_some.load(std::memory_order_relaxed) > 0 && g_fail_skip.fetch_sub(1, std::memory_order_relaxed) <= 0) {
+        g_fail_some.fetch_sub(1, std::memory_order_relaxed);
+        fail = true;
+    }
+    if (fail) {
         set_error("device allocation of %zu bytes failed (injected)", bytes);
         return SJ_ERR_OOM;
     }
@@ -292,13 +302,15 @@ static int copy_pages(const T* const* pages, int n_pages, int64_t page_pairs, in
 
 // The recheck queue of a join (queue_entries).  When memory is short, a
 // tensor-core filter makes do with the pairs' own share: the tile kernel deals
-// with the records past the queue.
+// with the records past the queue.  `small`: that share at once.
 static int alloc_queue(int2** band, unsigned long long* cap, int kernel, unsigned long long ev, bool dist,
-                       cudaStream_t s) {
+                       cudaStream_t s, bool small = false) {
     *cap = queue_entries(kernel, ev, dist);
-    int st = dev_alloc_t(band, (size_t)*cap, s);
     const unsigned long long least = std::max<unsigned long long>(ev / (dist ? 8 : 64), 1ull << 20);
+    if (small) *cap = std::min(*cap, least);
+    int st = dev_alloc_t(band, (size_t)*cap, s);
     if (st == SJ_ERR_OOM && *cap > least) {
+        clear_error();
         *cap = least;
         st = dev_alloc_t(band, (size_t)least, s);
     }
@@ -357,6 +369,13 @@ int sj_index_phase_ms(sj_handle h, double* device_ms, double* host_ms) {
         if (host_ms) host_ms[k] = h->phase_host_ms[k];
     }
     return SJ_OK;
+}
+
+int64_t sj_debug_fail_some_allocations(int64_t after, int64_t count) {
+    const long long due = g_fail_some.exchange(0, std::memory_order_relaxed);
+    g_fail_skip.store(after < 0 ? 0 : after, std::memory_order_relaxed);
+    g_fail_some.store(count < 0 ? 0 : count, std::memory_order_relaxed);
+    return due;
 }
 
 void sj_debug_fail_allocations(int64_t after) { g_fail_after.store(after < 0 ? -1 : after, std::memory_order_relaxed); }
@@ -1329,6 +1348,7 @@ int join_batch_impl(const double* const* pts, const int64_t* n, const int32_t* d
         std::vector<BatchJoin> hbj(groups.size());
         std::vector<JoinOut> jos(groups.size());
         std::vector<int2*> bands(groups.size(), nullptr);
+        bool small_queues = false;
         for (size_t gi = 0; gi < groups.size() && st == SJ_OK; ++gi) {
             BatchGroup& g = *groups[gi];
             BatchJoin bj{};
@@ -1354,7 +1374,19 @@ int join_batch_impl(const double* const* pts, const int64_t* n, const int32_t* d
             if (ix->n_items == 0) continue;
             const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
             unsigned long long band_cap = 0;
-            if ((st = alloc_queue(&bands[gi], &band_cap, ix->kernel, ev, dist, s)) != SJ_OK) break;
+            st = alloc_queue(&bands[gi], &band_cap, ix->kernel, ev, dist, s, small_queues);
+            if (st == SJ_ERR_OOM && !small_queues) {  // the groups' queues side by side: all of them small
+                clear_error();
+                for (int2*& b : bands) {
+                    dev_free(b, s);
+                    b = nullptr;
+                }
+                small_queues = true;
+                st = SJ_OK;
+                gi = (size_t)-1;  // (from the first group again)
+                continue;
+            }
+            if (st != SJ_OK) break;
             jos[gi].band = bands[gi];
             jos[gi].band_cap = band_cap;
             jos[gi].batch = dbj + gi;

@@ -1,0 +1,128 @@
+"""Scratch that makes do with less when memory is short: one allocation (or two
+in a row) of a call fails and those after it succeed (injected on the host).
+Each attempt either ends with SJ_ERR_OOM and nothing kept, or returns the
+oracle's result with no error message left behind; the ones that have a smaller
+form to fall back on must succeed."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2209_11287_gb300 import binding
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    yield
+    binding.sj_debug_fail_some_allocations(0, 0)
+
+
+def _sweep(run, check, count=1):
+    """Fails the allocations k .. k + count - 1 of the call for k = 0, 1, ...
+    up to its last one: those it survived."""
+    check(run()[0])
+    torch.cuda.synchronize()
+    base = binding.sj_debug_live_allocations()
+    survived = []
+    for k in range(400):
+        binding.sj_debug_fail_some_allocations(k, count)
+        try:
+            out, message = run()
+        except binding.SimJoinError as e:
+            assert e.status == binding.SJ_ERR_OOM, (k, e)
+            out = None
+        finally:
+            due = binding.sj_debug_fail_some_allocations(0, 0)
+        torch.cuda.synchronize()
+        assert binding.sj_debug_live_allocations() == base, k
+        if out is not None:
+            check(out)
+            if due > 0:
+                return survived
+            assert message == "", (k, message)
+            survived.append(k)
+    raise AssertionError("the call never ran to its end")
+
+
+def _join(pts, eps, **opt):
+    r = binding.sj_join(pts, eps, binding.sj_default_options(**opt))
+    message = binding.sj_last_error_message()
+    out = binding.sj_result_copy(r)
+    binding.sj_result_free(r)
+    return out, message
+
+
+def _points(n, seed):
+    g = np.random.Generator(np.random.PCG64(seed))
+    return g.random((n, 2))
+
+
+def _keys(pairs):
+    return binding.pairs_to_keys(pairs)
+
+
+@pytest.mark.parametrize("emit", [False, True], ids=["pairs", "distances"])
+def test_record_queue_of_one_join(emit):
+    x, eps = _points(5001, 1), 0.04
+    ref, rd = oracle.join(x, eps, with_dist=True)
+    pts = torch.from_numpy(x).cuda()
+
+    def check(out):
+        key = (out[0][:, 0].astype(np.int64) << 32) | out[0][:, 1]
+        order = np.argsort(key)
+        assert np.array_equal(key[order], ref)
+        if emit:
+            assert np.array_equal(out[1][order], rd)
+
+    # no index, one query an item: more than 2^23 evaluations, so the queue asks for more than its least size
+    survived = _sweep(lambda: _join(pts, eps, kernel="filter_fp16x2", indexed_dims=-1, queries_per_item=1,
+                                    emit_distances=int(emit), max_pairs_hint=1 << 20), check)
+    assert emit or len(survived) == 1
+
+
+def test_record_queue_of_a_join_to_host():
+    x, eps = _points(5001, 2), 0.04
+    ref = oracle.join(x, eps)
+    pts = torch.from_numpy(x).cuda()
+
+    def run():
+        h = binding.sj_build_index(pts, eps, binding.sj_default_options(kernel="filter_fp16x2", indexed_dims=-1,
+                                                                        queries_per_item=1))
+        try:
+            out = np.empty((ref.size, 2), dtype=np.int32)
+            cnt, _ = binding.sj_self_join_to_host(h, out, 1 << 20)
+            return out[:cnt], binding.sj_last_error_message()
+        finally:
+            binding.sj_destroy(h)
+
+    assert len(_sweep(run, lambda out: np.testing.assert_array_equal(_keys(out), ref))) == 1
+
+
+def test_record_queues_of_a_batch():
+    # two tensor groups: where not even the least queue of the second fits
+    # beside the first one's, both are taken at their least size
+    g = np.random.Generator(np.random.PCG64(3))
+    sets = [(g.random((5001, 2)), 0.04), (g.random((5001, 9)), 0.3)]
+    refs = [oracle.join(x, e) for x, e in sets]
+    pts = [torch.from_numpy(x).cuda() for x, _ in sets]
+
+    def run():
+        res = binding.sj_join_batch(pts, [e for _, e in sets], binding.sj_default_options(
+            kernel="filter_fp16x2", indexed_dims=-1, queries_per_item=1, max_pairs_hint=1 << 22))
+        message = binding.sj_last_error_message()
+        out = [binding.sj_result_copy(r)[0] for r in res]
+        for r in res:
+            binding.sj_result_free(r)
+        return out, message
+
+    def check(out):
+        for p, ref in zip(out, refs):
+            assert np.array_equal(_keys(p), ref)
+
+    assert len(_sweep(run, check)) >= 2
+    assert len(_sweep(run, check, count=2)) >= 1
