@@ -2006,18 +2006,32 @@ int build_index(Index* ix, const double* pts) {
     const int64_t Mc = (int64_t)M;
     ep.local_mask = ~0ull;
     // runs in fixed slots where they take at most 512 MB: one pass, one read-back
-    // of the totals at the end (the items within their upper bound)
+    // of the totals at the end (the items within their upper bound); packed
+    // below, at their number, where there is no room for that
     int64_t slots = 2;  // 3^(m-1) runs, one more when the self offset splits
     for (int k = 1, p3 = 1; k < ix->m; ++k) slots = (p3 *= 3) + 1;
-    if (ix->m > 0 && Mc * slots * (int64_t)sizeof(Run) <= (int64_t(512) << 20)) {
+    const int64_t items_cap = Mc + n / qmax + 1;
+    bool fixed = ix->m > 0 && Mc * slots * (int64_t)sizeof(Run) <= (int64_t(512) << 20);
+    if (fixed) {
+        int st = dev_alloc_t(&ix->runs, (size_t)(Mc * slots), s);
+        if (st == SJ_OK) st = dev_alloc_t(&ix->items, (size_t)items_cap, s);
+        if (st == SJ_ERR_OOM) {
+            clear_error();
+            dev_free(ix->runs, s);
+            dev_free(ix->items, s);
+            ix->runs = nullptr;
+            ix->items = nullptr;
+            fixed = false;
+        } else if (st != SJ_OK) {
+            return st;
+        }
+    }
+    if (fixed) {
         uint32_t* item_off = nullptr;
         EnumTotals* dtot = nullptr;
         SJ_TRY(tmp.alloc(&item_off, (size_t)Mc));
         SJ_TRY(tmp.alloc(&dtot, 1));
         SJ_CK(cudaMemsetAsync(dtot, 0, sizeof(EnumTotals), s));
-        const int64_t items_cap = Mc + n / qmax + 1;
-        SJ_TRY(dev_alloc_t(&ix->runs, (size_t)(Mc * slots), s));
-        SJ_TRY(dev_alloc_t(&ix->items, (size_t)items_cap, s));
         SJ_TRY((scan_exclusive<uint32_t, LoadCellItems>(LoadCellItems{ix->cell_start, (uint32_t)qmax}, item_off, Mc, false, s)));
         const unsigned blocks = (unsigned)std::min<int64_t>((Mc + 127) / 128, (int64_t)device_sm_count(ix->device) * 16);
         k_enum_cells<<<blocks, 128, 0, s>>>(ep, ix->cell_key, ix->cell_start, Mc, item_off, (uint32_t)slots, ix->runs,

@@ -126,3 +126,27 @@ def test_record_queues_of_a_batch():
 
     assert len(_sweep(run, check)) >= 2
     assert len(_sweep(run, check, count=2)) >= 1
+
+
+def test_runs_of_a_sparse_key_space():
+    """The runs in fixed slots and the items beside them: packed runs instead."""
+    g = np.random.Generator(np.random.PCG64(4))
+    x, eps = g.random((6000, 3)), 0.004
+    ref = oracle.join(x, eps)
+    pts = torch.from_numpy(x).cuda()
+    infos = []
+
+    def run():
+        h = binding.sj_build_index(pts, eps, binding.sj_default_options(kernel="filter_f32"))
+        message = binding.sj_last_error_message()
+        due = binding.sj_debug_fail_some_allocations(0, 0)  # (the build's allocations only)
+        r = binding.sj_self_join(h)
+        out = binding.sj_result_copy(r)[0]
+        infos.append(binding.sj_index_info(h))
+        binding.sj_result_free(r)
+        binding.sj_destroy(h)
+        binding.sj_debug_fail_some_allocations(1 << 30, due)
+        return out, message
+
+    assert len(_sweep(run, lambda out: np.testing.assert_array_equal(_keys(out), ref))) >= 2
+    assert all(i == infos[0] for i in infos)
