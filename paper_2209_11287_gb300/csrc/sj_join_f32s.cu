@@ -611,8 +611,17 @@ bool f32s_supported(const Index* ix, int emit_dist) {
 int launch_join_f32s(Index* ix, const JoinOut& out) {
     JoinParams p = make_join_params(ix, out, 0);
     Scratch tmp(ix->stream);  // (released after the launches that use it, stream-ordered)
-    const SparseUse sparse = f32r_use(ix, p);
-    if (sparse == SparseUse::few_queries) SJ_TRY(tmp.alloc(&p.big_items, (size_t)ix->n_items));
+    SparseUse sparse = f32r_use(ix, p);
+    if (sparse == SparseUse::few_queries) {
+        const int st = tmp.alloc(&p.big_items, (size_t)ix->n_items);
+        if (st == SJ_ERR_OOM) {  // no room for the list: k_join_f32s takes all items
+            clear_error();
+            p.big_items = nullptr;
+            sparse = SparseUse::none;
+        } else if (st != SJ_OK) {
+            return st;
+        }
+    }
     if (sparse != SparseUse::none) SJ_TRY(launch_join_f32r(ix, p));
     if (sparse == SparseUse::all) return SJ_OK;
     switch (ix->dp) {

@@ -150,3 +150,32 @@ def test_runs_of_a_sparse_key_space():
 
     assert len(_sweep(run, lambda out: np.testing.assert_array_equal(_keys(out), ref))) >= 2
     assert all(i == infos[0] for i in infos)
+
+
+def test_list_of_the_items_of_many_queries():
+    """Crowded cells among single points: without the list that the two FP32
+    filters share the items by, one of them takes all."""
+    g = np.random.Generator(np.random.PCG64(5))
+    x = g.random((7001, 3))
+    x[:2300] = 0.5 + 0.02 * (g.random((2300, 3)) - 0.5) + 0.25 * g.integers(0, 2, (2300, 1))
+    eps = (0.3 / 7001) ** (1.0 / 3)
+    ref = oracle.join(x, eps)
+    h = binding.sj_build_index(torch.from_numpy(x).cuda(), eps,
+                               binding.sj_default_options(kernel="filter_f32", max_pairs_hint=1 << 22))
+
+    def run():
+        launches = binding.sj_kernel_launches()
+        r = binding.sj_self_join(h)
+        message = binding.sj_last_error_message()
+        kernels.append(binding.sj_kernel_launches() - launches)
+        out = binding.sj_result_copy(r)[0]
+        binding.sj_result_free(r)
+        return out, message
+
+    kernels = []
+    try:
+        survived = _sweep(run, lambda out: np.testing.assert_array_equal(_keys(out), ref))
+    finally:
+        binding.sj_destroy(h)
+    assert len(survived) == 1
+    assert kernels[0] == kernels[1] + 1 == kernels[2]  # (two tile kernels where the list is there)
