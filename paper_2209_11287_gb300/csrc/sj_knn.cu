@@ -79,13 +79,16 @@ struct __align__(16) KnnEntry {
 // kNN from a join: bucket sizes (self pairs left out) and every pair's place
 // in its bucket, so the bucketing below needs no second atomic per pair (9.4 M
 // pairs, both kernels: 213 us with an atomic in each and two stores per pair,
-// 185 us so) ...
+// 185 us so) ...  These take 20 bytes a pair; where that finds no room, the
+// entries are split (12 bytes a pair: place null, one atomic more).
 __global__ void k_knn_degree(const int2* __restrict__ pairs, long long count, uint32_t* deg,
                              uint32_t* __restrict__ place) {
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < count;
          p += (long long)gridDim.x * blockDim.x) {
         const int2 e = pairs[p];
-        if (e.x != e.y) place[p] = atomicAdd(&deg[e.x], 1u);
+        if (e.x == e.y) continue;
+        const uint32_t at = atomicAdd(&deg[e.x], 1u);
+        if (place) place[p] = at;
     }
 }
 
@@ -100,6 +103,33 @@ __global__ void k_knn_bucket(const int2* __restrict__ pairs, const double* __res
         *reinterpret_cast<int4*>(nb + off[e.x] + place[p]) = make_int4((int)d, (int)(d >> 32), e.y, 0);
     }
 }
+
+__global__ void k_knn_bucket_split(const int2* __restrict__ pairs, const double* __restrict__ dist, long long count,
+                                   const uint32_t* __restrict__ off, uint32_t* cursor, int32_t* nb_idx,
+                                   double* nb_dist) {
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < count;
+         p += (long long)gridDim.x * blockDim.x) {
+        const int2 e = pairs[p];
+        if (e.x == e.y) continue;
+        const uint32_t s = off[e.x] + atomicAdd(&cursor[e.x], 1u);
+        nb_idx[s] = e.y;
+        nb_dist[s] = dist[p];
+    }
+}
+
+// Where the selection reads its entries (as KnnEntry's four words).
+struct KnnWhole {
+    const int4* e;
+    __device__ __forceinline__ int4 operator[](uint32_t s) const { return e[s]; }
+};
+struct KnnSplit {
+    const int32_t* idx;
+    const double* dist;
+    __device__ __forceinline__ int4 operator[](uint32_t s) const {
+        const long long d = __double_as_longlong(dist[s]);
+        return make_int4((int)d, (int)(d >> 32), idx[s], 0);
+    }
+};
 
 // ... and, one warp per point, its k smallest by (distance, index).
 //
@@ -129,15 +159,15 @@ constexpr int kKnnCut = kKnnList - 64;   // largest k the list is cut back to
 constexpr int kKnnEarly = 24;
 constexpr int kKnnWarps = 8;
 
+template <typename Src>
 __global__ void __launch_bounds__(32 * kKnnWarps) k_knn_select(int64_t n, int k, const uint32_t* __restrict__ off,
-                                                               const KnnEntry* __restrict__ nb, int32_t* idx_out,
-                                                               double* dist_out, int32_t* found_out) {
+                                                               const Src src, int32_t* idx_out, double* dist_out,
+                                                               int32_t* found_out) {
     __shared__ int4 s_list[kKnnWarps][kKnnList];
     const int lane = threadIdx.x & 31;
     const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (i >= n) return;
     const uint32_t a = off[i], b = off[i + 1];
-    const int4* __restrict__ src = reinterpret_cast<const int4*>(nb);
     const int found = (int)min(b - a, (uint32_t)k);
     if (b - a <= (uint32_t)kKnnList || k <= kKnnCut) {
         int4* list = s_list[threadIdx.x >> 5];
@@ -276,15 +306,29 @@ extern "C" int sj_knn_from_join(const sj_result* r, int64_t n, int32_t k, int32_
     int32_t *oi = nullptr, *of = nullptr;
     uint32_t *deg = nullptr, *off = nullptr, *place = nullptr;
     KnnEntry* nb = nullptr;
-    double* od = nullptr;
+    int32_t* nb_idx = nullptr;
+    double *nb_dist = nullptr, *od = nullptr;
     const size_t slots = (size_t)std::max<long long>(count, 1);
     SJ_TRY(tmp.alloc(&deg, (size_t)n));
     SJ_TRY(tmp.alloc(&off, (size_t)n + 1));
-    SJ_TRY(tmp.alloc(&place, slots));
-    SJ_TRY(tmp.alloc(&nb, slots));
     SJ_TRY(tmp.alloc(&oi, (size_t)n * k));
     SJ_TRY(tmp.alloc(&od, (size_t)n * k));
     SJ_TRY(tmp.alloc(&of, (size_t)n));
+    int st = dev_alloc_t(&nb, slots, s);
+    if (st == SJ_OK) st = dev_alloc_t(&place, slots, s);
+    if (st == SJ_ERR_OOM) {  // the split entries then
+        clear_error();
+        dev_free(nb, s);
+        nb = nullptr;
+        SJ_TRY(tmp.alloc(&nb_idx, slots));
+        SJ_TRY(tmp.alloc(&nb_dist, slots));
+    } else if (st != SJ_OK) {
+        dev_free(nb, s);
+        return st;
+    } else {
+        tmp.ptrs.push_back(nb);
+        tmp.ptrs.push_back(place);
+    }
     SJ_CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(uint32_t), s));
     if (count > 0) {
         k_knn_degree<<<grid_for(count, dev), 256, 0, s>>>(pairs, count, deg, place);
@@ -293,11 +337,20 @@ extern "C" int sj_knn_from_join(const sj_result* r, int64_t n, int32_t k, int32_
     }
     SJ_TRY(scan_exclusive_u32_total(deg, off, n, s));  // off[n]: the total
     if (count > 0) {
-        k_knn_bucket<<<grid_for(count, dev), 256, 0, s>>>(pairs, dist, count, off, place, nb);
+        if (nb) {
+            k_knn_bucket<<<grid_for(count, dev), 256, 0, s>>>(pairs, dist, count, off, place, nb);
+        } else {
+            SJ_CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(uint32_t), s));  // the buckets' cursors
+            k_knn_bucket_split<<<grid_for(count, dev), 256, 0, s>>>(pairs, dist, count, off, deg, nb_idx, nb_dist);
+        }
         note_launch();
         SJ_CK(cudaGetLastError());
     }
-    k_knn_select<<<(unsigned)((n + kKnnWarps - 1) / kKnnWarps), 32 * kKnnWarps, 0, s>>>(n, k, off, nb, oi, od, of);
+    const unsigned gs = (unsigned)((n + kKnnWarps - 1) / kKnnWarps);
+    if (nb)
+        k_knn_select<<<gs, 32 * kKnnWarps, 0, s>>>(n, k, off, KnnWhole{reinterpret_cast<const int4*>(nb)}, oi, od, of);
+    else
+        k_knn_select<<<gs, 32 * kKnnWarps, 0, s>>>(n, k, off, KnnSplit{nb_idx, nb_dist}, oi, od, of);
     note_launch();
     SJ_CK(cudaGetLastError());
     SJ_CK(cudaMemcpyAsync(idx_out, oi, (size_t)n * k * sizeof(int32_t), cudaMemcpyDefault, s));

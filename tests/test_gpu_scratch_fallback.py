@@ -179,3 +179,24 @@ def test_list_of_the_items_of_many_queries():
         binding.sj_destroy(h)
     assert len(survived) == 1
     assert kernels[0] == kernels[1] + 1 == kernels[2]  # (two tile kernels where the list is there)
+
+
+@pytest.mark.parametrize("k", [4, 30, 200])
+def test_entries_of_the_knn_selection(k):
+    """Without room for 16 bytes a pair and its place: 12 bytes a pair."""
+    x, eps = _points(3000, 6), 0.12
+    r = binding.sj_join(torch.from_numpy(x).cuda(), eps, binding.sj_default_options(emit_distances=1))
+    want = binding.sj_knn_from_join(r, x.shape[0], k)
+
+    def run():
+        out = binding.sj_knn_from_join(r, x.shape[0], k)
+        return out, binding.sj_last_error_message()
+
+    def check(out):
+        for a, b in zip(out, want):
+            assert np.array_equal(a, b)
+
+    try:
+        assert len(_sweep(run, check)) == 2
+    finally:
+        binding.sj_result_free(r)
