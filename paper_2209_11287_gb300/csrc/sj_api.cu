@@ -303,9 +303,10 @@ static int copy_pages(const T* const* pages, int n_pages, int64_t page_pairs, in
 // The recheck queue of a join (queue_entries).  When memory is short, a
 // tensor-core filter makes do with the pairs' own share: the tile kernel deals
 // with the records past the queue.  `small`: that share at once.
-static int alloc_queue(int2** band, unsigned long long* cap, int kernel, unsigned long long ev, bool dist,
-                       cudaStream_t s, bool small = false) {
-    *cap = queue_entries(kernel, ev, dist);
+static int alloc_queue(int2** band, unsigned long long* cap, const Index* ix, bool dist, cudaStream_t s,
+                       bool small = false) {
+    const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
+    *cap = queue_entries(ix->kernel, ev, (double)ix->n / (double)std::max<int64_t>(ix->n_items, 1), dist);
     const unsigned long long least = std::max<unsigned long long>(ev / (dist ? 8 : 64), 1ull << 20);
     if (small) *cap = std::min(*cap, least);
     int st = dev_alloc_t(band, (size_t)*cap, s);
@@ -570,11 +571,10 @@ static int run_join(sj_index* ix, ResultImpl* ri, int64_t page_pairs, bool dist,
     }
     // deferred-recheck queue: band pairs (and, with distances, every
     // maybe-in pair); pairs past its end are re-decided in place
-    const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
     Scratch tmp(s);
     int2* band = nullptr;
     unsigned long long band_cap = 0;
-    SJ_TRY(alloc_queue(&band, &band_cap, ix->kernel, ev, dist, s));
+    SJ_TRY(alloc_queue(&band, &band_cap, ix, dist, s));
     tmp.ptrs.push_back(band);
     JoinOut jo;
     jo.out_pairs = reinterpret_cast<int2*>(ri->block);
@@ -653,7 +653,6 @@ int sj_self_join_to_host(sj_handle h, int32_t* host_pairs, int64_t host_capacity
     sj_index* ix = h;
     cudaStream_t s = ix->stream;
     const int64_t n_items = ix->n_items;
-    const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
     unsigned long long band_cap = 0;
     int2* pool[2] = {nullptr, nullptr};
     int2* band = nullptr;
@@ -662,7 +661,7 @@ int sj_self_join_to_host(sj_handle h, int32_t* host_pairs, int64_t host_capacity
     int st = SJ_OK;
     if ((st = dev_alloc_t(&pool[0], (size_t)device_pairs, s)) == SJ_OK &&
         (st = dev_alloc_t(&pool[1], (size_t)device_pairs, s)) == SJ_OK)
-        st = alloc_queue(&band, &band_cap, ix->kernel, ev, false, s);
+        st = alloc_queue(&band, &band_cap, ix, false, s);
     if (st == SJ_OK) {
         cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
         for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
@@ -1372,9 +1371,8 @@ int join_batch_impl(const double* const* pts, const int64_t* n, const int32_t* d
             hbj[gi] = bj;
             Index* ix = &g.ix;
             if (ix->n_items == 0) continue;
-            const unsigned long long ev = (unsigned long long)std::max<int64_t>(ix->n_evaluated, 1);
             unsigned long long band_cap = 0;
-            st = alloc_queue(&bands[gi], &band_cap, ix->kernel, ev, dist, s, small_queues);
+            st = alloc_queue(&bands[gi], &band_cap, ix, dist, s, small_queues);
             if (st == SJ_ERR_OOM && !small_queues) {  // the groups' queues side by side: all of them small
                 clear_error();
                 for (int2*& b : bands) {

@@ -277,17 +277,19 @@ int launch_recheck(Index* ix, const JoinOut& out, int emit_dist);
 int launch_resolve(Index* ix, const JoinOut& out, int emit_dist);
 // Entries (8 bytes) of the recheck queue of a join of `ev` evaluations.  A
 // tensor-core filter keeps its 16-byte records there, one per candidate and 32
-// query columns with a maybe-in pair: room for ev / 16 of them, at most 2 GB or
-// the pairs' own share, which is a record of every 128 evaluations (16 with
-// distances).  More come of items of few queries (up to one per evaluation) and,
-// above 2^31 evaluations, of joins with a pair in most blocks of 32: the tile
+// query columns with a maybe-in pair: room for one per min(per_item, 16)
+// evaluations (per_item: queries of a work item on average; an item of fewer
+// than 32 has at most a record per candidate), at most 2 GB or the pairs' own
+// share, which is a record of every 128 evaluations (16 with distances).  Above
+// 2^31 evaluations a join with a pair in most blocks of 32 has more: the tile
 // kernel deals with the records past the queue.
-inline unsigned long long queue_entries(int kernel, unsigned long long ev, bool dist) {
+inline unsigned long long queue_entries(int kernel, unsigned long long ev, double per_item, bool dist) {
     const unsigned long long small = ev / (dist ? 8 : 64), least = 1ull << 20;
     unsigned long long cap = small;
     if (is_tensor_kernel(kernel)) {
         const unsigned long long most = small > (1ull << 28) ? small : 1ull << 28;
-        cap = ev / 8 < most ? ev / 8 : most;
+        const double want = 2.0 * (double)ev / (per_item < 1.0 ? 1.0 : per_item > 16.0 ? 16.0 : per_item);
+        cap = want < (double)most ? (unsigned long long)want : most;
         if (cap < small) cap = small;
         return cap > least ? cap : least;  // (room for whole reservations however few the evaluations)
     }
