@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(32 * kResolveWarps, kResolveBlocks) k_resolve(
     auto deal = [&](bool live, int2 e) {
         const int32_t qs = (int32_t)((uint32_t)e.x & ~kMirrorBit), cs = (int32_t)((uint32_t)e.y & ~kMirrorBit);
         live = live && SJ_BOUND(P, qs < P.n_points && cs < P.n_points, 41);
-        const bool certain = !EMIT && e.x < 0;
+        const bool certain = e.x < 0;
         int nout = 0, gid = 0;
         int32_t qid = 0, cid = 0;
         double dist = 0.0;
@@ -84,17 +84,18 @@ __global__ void __launch_bounds__(32 * kResolveWarps, kResolveBlocks) k_resolve(
             qid = P.perm[qs];
             cid = P.perm[cs];
             const int li = inst_of ? inst_of[qs] : 0;
-            bool in = certain;
+            bool in = certain, exact = EMIT && certain;  // (exact: the binary64 sum is needed)
+            if (EMIT || !certain) ++decided;
             if (!certain) {
-                ++decided;
                 const float s32 = refine_sq<DP>(Y + (int64_t)qs * DP, Y + (int64_t)cs * DP);
                 const float2 r = inst_of ? P.batch->inst_refine[li] : make_float2(P.refine_out, P.refine_in);
                 in = s32 < r.y;
-                if (EMIT ? !(s32 > r.x) : !in && !(s32 > r.x)) {
-                    const double s = direct_sq(P.xs + (int64_t)qs * DP, P.xs + (int64_t)cs * DP, P.d);
-                    in = s <= (inst_of ? P.batch->inst_e2[li] : P.e2);
-                    if (EMIT && in) dist = sqrt(s);
-                }
+                exact = (EMIT || !in) && !(s32 > r.x);
+            }
+            if (exact) {
+                const double s = direct_sq(P.xs + (int64_t)qs * DP, P.xs + (int64_t)cs * DP, P.d);
+                in = s <= (inst_of ? P.batch->inst_e2[li] : P.e2);
+                if (EMIT && in) dist = sqrt(s);
             }
             if (in) nout = e.y < 0 && cs != qs ? 2 : 1;
             if (inst_of) {
@@ -150,13 +151,21 @@ __global__ void __launch_bounds__(32 * kResolveWarps, kResolveBlocks) k_resolve(
     // 96 joins in one batch: blocks a grid apart 6.52 ms, runs of 4 6.22, 16
     // 6.19, 64 6.17; one join of the 16-D mixture 2.64 / 2.67 / 2.67 / 2.77 ms,
     // long runs leave warps idle.
-    const unsigned long long warps = (unsigned long long)gridDim.x * kResolveWarps, blocks = (count + 31) / 32;
+    // Few records are spread over all warps in blocks of fewer (a block's pairs
+    // are dealt with 32 at a time, one after another).  4,000 x 64-D points with
+    // distances, 61,000 pairs, filter and this kernel: 188 us with blocks of 32
+    // and every pair in binary32 first, 128 so and with the certain ones in
+    // binary64 at once.
+    const unsigned long long warps = (unsigned long long)gridDim.x * kResolveWarps;
+    int size = 32;  // records of a block
+    while (size > 8 && count < warps * (unsigned)(size / 2)) size >>= 1;
+    const unsigned long long blocks = (count + (unsigned)size - 1) / (unsigned)size;
     const unsigned long long run = min((unsigned long long)kResolveRun, max(1ull, blocks / (2 * warps)));
     int of_list = -1;  // batch: the instance of the waiting pairs
     unsigned long long r = (unsigned long long)blockIdx.x * kResolveWarps + wid, k_run = 0;
     for (; r * run + k_run < blocks; k_run + 1 < run ? ++k_run : (k_run = 0, r += warps)) {
-        const unsigned long long b = (r * run + k_run) * 32;
-        const int4 e = b + lane < count ? records[b + lane] : make_int4(0, 0, 0, 0);
+        const unsigned long long b = (r * run + k_run) * (unsigned)size;
+        const int4 e = lane < size && b + lane < count ? records[b + lane] : make_int4(0, 0, 0, 0);
         if (inst_of) {  // what waits of another instance goes first, so that a warp of pairs has one
             const int cs = (int)((uint32_t)e.w & ~kMirrorBit);
             const unsigned some = __ballot_sync(0xffffffffu, e.x != 0);
