@@ -44,7 +44,7 @@ constexpr int cc_warps() {
     return sizeof(WS) * 4 <= 46 * 1024 ? 4 : sizeof(WS) * 2 <= 46 * 1024 ? 2 : 1;
 }
 
-template <typename T, int DP, int TC, bool EMIT, int RUNS>
+template <typename T, int DP, int TC, bool EMIT, int RUNS, bool PRUNE>
 struct CcWarpSmem {
     ItemSmem<T, DP, RUNS> it;
     int32_t cj[EMIT ? 32 * TC : 1];    // sorted position of each candidate slot (with distances)
@@ -55,12 +55,12 @@ struct CcWarpSmem {
     int2 stage[kStage];
     double sdist[EMIT ? kStage : 1];
     double scq[DP >= 16 ? kQMax : 1];  // short-circuit: each query's w
-    // d <= 8: candidates kept by the bounding-box prune (position, run flag),
-    // and the box of the item's queries
+    // candidates kept by the bounding-box prune (position, run flag), and the
+    // box of the item's queries
     static constexpr uint32_t RING = 32 * TC - 1 + 64 <= 128 ? 128 : 256;
-    int32_t ring_j[DP <= 8 ? RING : 1];
-    uint8_t ring_f[DP <= 8 ? RING : 1];
-    float blo[DP <= 8 ? DP : 1], bhi[DP <= 8 ? DP : 1];
+    int32_t ring_j[PRUNE ? RING : 1];
+    uint8_t ring_f[PRUNE ? RING : 1];
+    float blo[PRUNE ? DP : 1], bhi[PRUNE ? DP : 1];
 };
 
 // Compaction step of the prune, d <= 8: candidates [v0, v0 + 64) of the item,
@@ -68,16 +68,17 @@ struct CcWarpSmem {
 // `cnt` entries from `head`.  The same lossless test as k_join_f32s
 // (f32s_gather: a lower bound of the squared distance to the box, every
 // operation rounded down, against the radius behind the certified "out"
-// threshold), here in front of the tiles with distances and the FP64 tile.
+// threshold), here in front of the tiles with distances and the FP64 tile where
+// cc_prune says so.
 // The latter's binary64 coordinates are rounded to binary32 for it, which its
 // radius allows for (fp64_prune_r2).  `r` is the lane's run cursor.
 // A radius of +inf keeps everything.  Returns the candidates dropped.  Measured,
 // FP64 tile with distances (200,000 uniform 4-D points, 64 neighbours, 9 queries
 // an item; FP64 pipe): 705 us over all candidates, 495 us behind the prune.
 template <typename T, int DP, int TC, bool EMIT, int RUNS>
-__device__ __forceinline__ uint32_t cc_gather(CcWarpSmem<T, DP, TC, EMIT, RUNS>& W, const JoinParams& P, float r2,
+__device__ __forceinline__ uint32_t cc_gather(CcWarpSmem<T, DP, TC, EMIT, RUNS, true>& W, const JoinParams& P, float r2,
                                               uint32_t C, uint32_t v0, int lane, int& r, uint32_t head, uint32_t& cnt) {
-    constexpr uint32_t RING = CcWarpSmem<T, DP, TC, EMIT, RUNS>::RING;
+    constexpr uint32_t RING = CcWarpSmem<T, DP, TC, EMIT, RUNS, true>::RING;
     const T* __restrict__ Y = static_cast<const T*>(P.y);
     ItemSmem<T, DP, RUNS>& S = W.it;
     int32_t jj[2];
@@ -266,34 +267,41 @@ __device__ __forceinline__ void emit_direct(WarpStage& st, const JoinParams& P, 
 }
 
 // Minimum resident CTAs per SM requested from the register allocator, and
-// candidates per lane, of the FP32 small-d tile with distances (d <= 8).
-// Measured behind the bounding-box prune (200,003 uniform 3-D points, 48
-// neighbours), tile-kernel time: 9 CTAs (56 registers, spills) 156 us, 8 152,
-// 7 150; without the prune 155.  Compile-time tuning constants.
+// candidates per lane, of the FP32 small-d tile with distances (d <= 8): it is
+// latency-bound, so it runs with 2 candidates per lane and 9 CTAs of 4 warps per
+// SM (at most 56 registers); behind the bounding-box prune, which takes more
+// registers, with 7 (200,003 uniform 3-D points, 48 neighbours: 9 CTAs, with
+// spills, 156 us, 8 152, 7 150; without the prune 155).  Compile-time tuning
+// constants.
 #ifndef SJ_CC_F32_MIN_BLOCKS
-#define SJ_CC_F32_MIN_BLOCKS 7
+#define SJ_CC_F32_MIN_BLOCKS 9
+#endif
+#ifndef SJ_CC_F32_PRUNE_MIN_BLOCKS
+#define SJ_CC_F32_PRUNE_MIN_BLOCKS 7
 #endif
 #ifndef SJ_CC_TC_SMALL_D
 #define SJ_CC_TC_SMALL_D 2
 #endif
-template <typename T, int DP>
+template <typename T, int DP, bool PRUNE>
 constexpr int cc_min_blocks() {
-    return std::is_same<T, float>::value && DP <= 8 ? SJ_CC_F32_MIN_BLOCKS : 1;
+    return !std::is_same<T, float>::value || DP > 8 ? 1 : PRUNE ? SJ_CC_F32_PRUNE_MIN_BLOCKS : SJ_CC_F32_MIN_BLOCKS;
 }
 
-template <typename T, int DP, int TC, bool EMIT, int NW, int RUNS>
-__global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(JoinParams P) {
+// PRUNE (d <= 8): the candidates pass the bounding-box prune first (cc_prune).
+template <typename T, int DP, int TC, bool EMIT, int NW, int RUNS, bool PRUNE>
+__global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join_cc(JoinParams P) {
     constexpr bool FUSED = DP <= 8;
+    static_assert(FUSED || !PRUNE, "the prune is for small dimensions");
     constexpr int KC = DP < 8 ? DP : 8;  // dims per register chunk (unfused path)
     constexpr int SLOTS = 32 * TC;
     static_assert(SLOTS <= 2048, "slot index must fit in 11 bits");
-    __shared__ CcWarpSmem<T, DP, TC, EMIT, RUNS> smem[NW];
+    __shared__ CcWarpSmem<T, DP, TC, EMIT, RUNS, PRUNE> smem[NW];
 
     const T* __restrict__ Y = static_cast<const T*>(P.y);
     const T* __restrict__ TO = static_cast<const T*>(P.thr_out);
     const T* __restrict__ TI = static_cast<const T*>(P.thr_in);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    CcWarpSmem<T, DP, TC, EMIT, RUNS>& W = smem[wid];
+    CcWarpSmem<T, DP, TC, EMIT, RUNS, PRUNE>& W = smem[wid];
     ItemSmem<T, DP, RUNS>& S = W.it;
     WarpStage st{W.stage, EMIT ? W.sdist : nullptr, 0, 0};
     BandQ bq{0, 0};
@@ -319,10 +327,7 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
             }
         }
 
-        float box_r2 = INFINITY;
-        if constexpr (FUSED) {  // the box of the queries (32 is a multiple of DP: a lane keeps to one dim)
-            // (a batched FP64 join has no radius that allows for the rounding)
-            box_r2 = std::is_same<T, double>::value && P.batch ? INFINITY : R.r2;
+        if constexpr (PRUNE) {  // the box of the queries (32 is a multiple of DP: a lane keeps to one dim)
             float bmin = INFINITY, bmax = -INFINITY;
             for (int i = lane; i < Q * DP; i += 32) {
                 const float v = (float)S.qy[i / DP][i % DP];
@@ -341,12 +346,12 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
             __syncwarp();
         }
         int run = 0;
-        uint32_t head = 0, cnt = 0, v0 = 0;  // the ring (d <= 8); candidates gathered
+        uint32_t head = 0, cnt = 0, v0 = 0;  // the ring; candidates gathered
         for (uint32_t base = 0;;) {
             uint32_t ns;  // candidates of this chunk
-            if constexpr (FUSED) {
+            if constexpr (PRUNE) {
                 while (v0 < C && cnt < (uint32_t)SLOTS) {
-                    const uint32_t out = cc_gather<T, DP, TC, EMIT, RUNS>(W, P, box_r2, C, v0, lane, run, head, cnt);
+                    const uint32_t out = cc_gather<T, DP, TC, EMIT, RUNS>(W, P, R.r2, C, v0, lane, run, head, cnt);
                     if constexpr (std::is_same<T, float>::value) pruned += (unsigned long long)out * (unsigned long long)Q;
                     v0 += 64u;
                 }
@@ -371,8 +376,8 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
                 ti[t] = T(INFINITY);
                 if (valid[t]) {
                     uint8_t fl;
-                    if constexpr (FUSED) {
-                        const uint32_t e = (head + (uint32_t)slot) & (CcWarpSmem<T, DP, TC, EMIT, RUNS>::RING - 1u);
+                    if constexpr (PRUNE) {
+                        const uint32_t e = (head + (uint32_t)slot) & (CcWarpSmem<T, DP, TC, EMIT, RUNS, true>::RING - 1u);
                         j[t] = W.ring_j[e];
                         fl = W.ring_f[e];
                     } else {
@@ -525,8 +530,8 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
             __syncwarp();
             }
             }
-            if constexpr (FUSED) {
-                head = (head + ns) & (CcWarpSmem<T, DP, TC, EMIT, RUNS>::RING - 1u);
+            if constexpr (PRUNE) {
+                head = (head + ns) & (CcWarpSmem<T, DP, TC, EMIT, RUNS, true>::RING - 1u);
                 cnt -= ns;
                 __syncwarp();
             } else {
@@ -542,11 +547,32 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP>()) k_join_cc(Joi
     if (lane == 0 && rechecked) atomicAdd(&P.counters[2], rechecked);
 }
 
-template <typename T, int DP, bool EMIT, int RUNS>
+// Whether a join's candidates pass the bounding-box prune: where items have more
+// than 140 candidates, so that it saves whole chunks (of 128 candidates in FP64,
+// 64 in FP32) and not slots of one, and in FP64 more than 300 evaluations, for
+// its own cost an item.  Planar cells keep 83% of their candidates, so padded
+// d = 2 goes without it, and so do joins without an index (the box of 16
+// arbitrary points spans everything) and batches (no radius per instance for the
+// FP64 tile).  Tile times without / with it, us, by candidates an item (200,000
+// points): FP64 3-D 75 196 / 233, 150 362 / 273, 718 1183 / 1000; 4-D 24 252 /
+// 325, 94 219 / 271, 175 337 / 267, 644 1028 / 717; 6-D 50 572 / 788, 149 (200
+// evaluations) 862 / 960, 265 (440) 1108 / 1025, 2026 6070 / 2547; clusters 4-D
+// 94 303 / 320, 295 664 / 578; 2-D 18 123 / 140, 355 626 / 625; 8-D without an
+// index 6468 / 7373.  FP64 with distances 4-D 24 263 / 412, 175 335 / 289.  FP32
+// with distances 3-D 39 91 / 102, 75 103 / 104, 150 150 / 144; 4-D 24 115 / 153,
+// 94 99 / 106, 175 102 / 99, 644 204 / 176; 6-D 50 296 / 334, 149 474 / 428,
+// 2026 766 / 565; 2-D 10 83 / 91, 76 206 / 197.
+inline bool cc_prune(const Index* ix, const JoinParams& p, bool fp64) {
+    if (p.batch || ix->m == 0 || ix->n_cells <= 0 || ix->dp == 2) return false;
+    const double n = (double)ix->n, ev = (double)ix->n_evaluated;
+    return ev > 140.0 * n && (!fp64 || ev > 300.0 * ((double)ix->n_cells + n / kQMax));
+}
+
+template <typename T, int DP, bool EMIT, int RUNS, bool PRUNE>
 inline int launch_dper(Index* ix, const JoinParams& p) {
     constexpr int TC = DP > 8 ? 2 : std::is_same<T, float>::value ? SJ_CC_TC_SMALL_D : 4;
-    constexpr int NW = cc_warps<CcWarpSmem<T, DP, TC, EMIT, RUNS>>();
-    auto kern = k_join_cc<T, DP, TC, EMIT, NW, RUNS>;
+    constexpr int NW = cc_warps<CcWarpSmem<T, DP, TC, EMIT, RUNS, PRUNE>>();
+    auto kern = k_join_cc<T, DP, TC, EMIT, NW, RUNS, PRUNE>;
     int per_sm = 0;
     SJ_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, 0));
     if (per_sm < 1) per_sm = 1;
@@ -565,10 +591,15 @@ inline int launch_dper(Index* ix, const JoinParams& p) {
 // bound by registers, so they keep the general capacity only.
 template <typename T, int DP, bool EMIT>
 inline int launch_dpe(Index* ix, const JoinParams& p) {
-    if constexpr (DP <= 8)
-        return ix->m <= 4 ? launch_dper<T, DP, EMIT, 28>(ix, p) : launch_dper<T, DP, EMIT, kMaxRuns>(ix, p);
-    else
-        return launch_dper<T, DP, EMIT, kMaxRuns>(ix, p);
+    if constexpr (DP <= 8) {
+        if constexpr (DP > 2)
+            if (cc_prune(ix, p, std::is_same<T, double>::value))
+                return ix->m <= 4 ? launch_dper<T, DP, EMIT, 28, true>(ix, p)
+                                  : launch_dper<T, DP, EMIT, kMaxRuns, true>(ix, p);
+        return ix->m <= 4 ? launch_dper<T, DP, EMIT, 28, false>(ix, p) : launch_dper<T, DP, EMIT, kMaxRuns, false>(ix, p);
+    } else {
+        return launch_dper<T, DP, EMIT, kMaxRuns, false>(ix, p);
+    }
 }
 
 // The tile launch for padded dimension DP.  The FP32 filter at DP <= 8
