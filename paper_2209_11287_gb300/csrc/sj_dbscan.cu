@@ -108,12 +108,15 @@ __device__ __forceinline__ void db_core_pairs(const int2 (&e)[kDbAhead], const u
     for (int u = 0; u < kDbAhead; ++u) take[u] = ((cx[u] >> (e[u].x & 31)) & (cy[u] >> (e[u].y & 31)) & 1u) != 0u;
 }
 
-__global__ void k_db_init(int64_t n, int32_t* parent, int32_t* border) {
+// (`status`: the error flag and the flag of k_db_core)
+__global__ void k_db_init(int64_t n, int32_t* parent, int32_t* border, int32_t* deg, unsigned long long* status) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) {
         parent[i] = (int32_t)i;
         border[i] = kNoLabel;
+        deg[i] = 0;
     }
+    if (i < 2) status[i] = 0;  // (n >= 1: at least one whole block)
 }
 
 __device__ __forceinline__ int32_t db_find(volatile int32_t* parent, int32_t x) {
@@ -265,9 +268,11 @@ __global__ void k_db_roots(int64_t n, const uint32_t* __restrict__ core, const i
 }
 
 __global__ void k_db_label(int64_t n, const uint32_t* __restrict__ core, const int32_t* __restrict__ parent,
-                           const int32_t* __restrict__ border, const uint32_t* __restrict__ rank, int32_t* labels) {
+                           const int32_t* __restrict__ border, const uint32_t* __restrict__ flag,
+                           const uint32_t* __restrict__ rank, int32_t* labels, unsigned long long* clusters) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
+    if (i == n - 1) *clusters = (unsigned long long)rank[i] + flag[i];
     int32_t l = -1;
     if (db_core(core, (int32_t)i))
         l = (int32_t)rank[parent[i]];
@@ -293,6 +298,14 @@ constexpr int kDbShare = 6;
 int db_stride(long long count, int64_t n) {
     return (int)std::max<long long>(1, std::min<long long>(count / (n * kDbShare), 1 << 20));
 }
+// Few pairs of few neighbours go straight to the union pass, where the rounds'
+// launches cost more than the walks (the whole call, with three read-backs
+// instead of one about 25 us longer than now, us, 0 / 1 / 3 rounds, by points x
+// neighbours, uniform 2-D to 4-D: 300 x 4 106 / 114 / 125, 3,000 x 4
+// 123 / 129 / 134, 10,000 x 4 170 / 170 / 158, 300,000 x 4 577 / 753 / 319; from
+// about 6 neighbours on three rounds are at least as fast at any size: 3,000 x
+// 11 170 / 182 / 132, 100,000 x 10 781 / 739 / 245, 300 x 42 137 / 131 / 124).
+int db_rounds(long long count, int64_t n) { return count < kDbShare * n && count < (1 << 15) ? 0 : kDbRounds; }
 
 }  // namespace
 
@@ -324,7 +337,7 @@ extern "C" int sj_dbscan(const sj_result* r, int64_t n, int32_t min_pts, int32_t
     Scratch tmp(s);
     int32_t *deg = nullptr, *parent = nullptr, *border = nullptr, *labels = nullptr;
     uint32_t *flag = nullptr, *core = nullptr;  // flag: n flags, then n + 1 ranks
-    unsigned long long* error = nullptr;        // the error flag, then the number of points that are not core
+    unsigned long long* error = nullptr;        // the error flag; whether a point is not core, later the clusters
     SJ_TRY(tmp.alloc(&deg, (size_t)n));
     SJ_TRY(tmp.alloc(&parent, (size_t)n));
     SJ_TRY(tmp.alloc(&border, (size_t)n));
@@ -333,10 +346,8 @@ extern "C" int sj_dbscan(const sj_result* r, int64_t n, int32_t min_pts, int32_t
     SJ_TRY(tmp.alloc(&core, (size_t)((n + 31) / 32)));
     SJ_TRY(tmp.alloc(&error, 2));
     uint32_t* rank = flag + n;
-    SJ_CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(int32_t), s));
-    SJ_CK(cudaMemsetAsync(error, 0, 2 * sizeof(unsigned long long), s));
     const unsigned gn = (unsigned)((n + 255) / 256);
-    k_db_init<<<gn, 256, 0, s>>>(n, parent, border);
+    k_db_init<<<gn, 256, 0, s>>>(n, parent, border, deg, error);
     note_launch();
     if (count > 0) {
         k_db_degree<<<grid_for(count, dev), kDbThreads, 0, s>>>(pairs, count, deg);
@@ -347,7 +358,7 @@ extern "C" int sj_dbscan(const sj_result* r, int64_t n, int32_t min_pts, int32_t
     if (count > 0) {
         // hooking rounds on a share of the pairs each, then all of them
         const int stride = db_stride(count, n);
-        const int rounds = stride > 1 ? kDbRounds : 1;
+        const int rounds = db_rounds(count, n);
         for (int r = 0; r < rounds; ++r) {
             k_db_hook<<<grid_for(count / stride, dev), kDbThreads, 0, s>>>(
                 pairs, count, stride, (int)((long long)r * stride / rounds), core, parent, parent);
@@ -366,20 +377,19 @@ extern "C" int sj_dbscan(const sj_result* r, int64_t n, int32_t min_pts, int32_t
     note_launch();
     SJ_CK(cudaGetLastError());
     SJ_TRY(scan_exclusive_u32(flag, rank, n, s));
-    k_db_label<<<gn, 256, 0, s>>>(n, core, parent, border, rank, labels);
+    k_db_label<<<gn, 256, 0, s>>>(n, core, parent, border, flag, rank, labels, error + 1);
     note_launch();
     SJ_CK(cudaGetLastError());
-    uint32_t last[2] = {0, 0};
-    unsigned long long err = 0;
-    SJ_CK(cudaMemcpyAsync(&last[0], rank + n - 1, 4, cudaMemcpyDeviceToHost, s));
-    SJ_CK(cudaMemcpyAsync(&last[1], flag + n - 1, 4, cudaMemcpyDeviceToHost, s));
-    SJ_CK(cudaMemcpyAsync(&err, error, sizeof err, cudaMemcpyDeviceToHost, s));
+    unsigned long long got[2] = {0, 0};  // the error flag, the number of clusters
+    void* hs = host_staging(sizeof got);  // pinned: a direct copy
+    SJ_CK(cudaMemcpyAsync(hs ? hs : got, error, sizeof got, cudaMemcpyDeviceToHost, s));
     SJ_CK(cudaMemcpyAsync(labels_out, labels, (size_t)n * sizeof(int32_t), cudaMemcpyDefault, s));
     SJ_CK(cudaStreamSynchronize(s));
-    if (err) {
+    if (hs) memcpy(got, hs, sizeof got);
+    if (got[0]) {
         set_error("a union-find update ran out of retries");
         return SJ_ERR_TIMEOUT;
     }
-    if (n_clusters) *n_clusters = (int64_t)last[0] + (int64_t)last[1];
+    if (n_clusters) *n_clusters = (int64_t)got[1];
     return SJ_OK;
 }
