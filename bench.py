@@ -280,8 +280,11 @@ def run_native(args):
         if host_out is not None:
             binding.sj_result_copy(r, host_out)
         count = sum(gather_counts(int(r.count), world, dev))
-        info = (count, int(r.n_candidates), int(r.n_evaluated), int(r.n_rechecked), int(r.reruns),
-                float(r.ms_tile), int(r.kernel))
+        evaluated = int(r.n_evaluated)
+        if int(r.kernel) == binding.KERNELS["fp64_fma"]:  # (reports what is scheduled)
+            evaluated -= binding.sj_index_last_pruned(h)
+        info = (count, int(r.n_candidates), evaluated, int(r.n_rechecked), int(r.reruns), float(r.ms_tile),
+                int(r.kernel))
         binding.sj_result_free(r)
         binding.sj_destroy(h)
         return info

@@ -176,6 +176,10 @@ SJ_API void sj_destroy(sj_handle h);
 SJ_API int sj_index_info(sj_handle h, int64_t* n_cells, int64_t* n_items, int32_t* m, int64_t* n_candidates,
                   int64_t* n_evaluated);
 
+/* Scheduled pair evaluations that the bounding-box prune removed from the last
+ * sj_self_join or sj_self_join_range of this index (0 for a NULL handle). */
+SJ_API int64_t sj_index_last_pruned(sj_handle h);
+
 /* ---- join -------------------------------------------------------------- */
 typedef struct sj_result {
     int64_t count;            /* |R|, exact */
@@ -192,7 +196,9 @@ typedef struct sj_result {
                                  index's scheduled evaluations less those the
                                  FP32 filter's bounding-box prune (padded
                                  d <= 8) removed; batched results and the FP64
-                                 tile report the scheduled evaluations */
+                                 tile report the scheduled evaluations (what
+                                 the prune removed from a join of the latter:
+                                 sj_index_last_pruned) */
     int64_t n_rechecked;      /* pairs the kernel's certified bound left open,
                                  re-decided by the direct form (behind a
                                  tensor-core filter in binary32 with a bound of

@@ -180,6 +180,8 @@ def load():
         lib.sj_debug_filter_dump.restype = ctypes.c_int
         lib.sj_index_perm.argtypes = [_vp, _vp]
         lib.sj_index_perm.restype = ctypes.c_int
+        lib.sj_index_last_pruned.argtypes = [_vp]
+        lib.sj_index_last_pruned.restype = _i64
         lib.sj_debug_fail_allocations.argtypes = [_i64]
         lib.sj_debug_fail_allocations.restype = None
         lib.sj_debug_fail_some_allocations.argtypes = [_i64, _i64]
@@ -289,6 +291,12 @@ def sj_index_info(handle) -> dict:
     _check(load().sj_index_info(handle, ctypes.byref(c), ctypes.byref(it), ctypes.byref(m), ctypes.byref(e),
                                 ctypes.byref(f)))
     return {"n_cells": c.value, "n_items": it.value, "m": m.value, "n_candidates": e.value, "n_evaluated": f.value}
+
+
+def sj_index_last_pruned(handle) -> int:
+    """Scheduled evaluations that the bounding-box prune removed from the
+    handle's last join."""
+    return int(load().sj_index_last_pruned(handle))
 
 
 def sj_self_join(handle) -> sj_result:

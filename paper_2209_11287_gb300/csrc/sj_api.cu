@@ -501,6 +501,8 @@ int sj_index_info(sj_handle h, int64_t* n_cells, int64_t* n_items, int32_t* m, i
     return SJ_OK;
 }
 
+int64_t sj_index_last_pruned(sj_handle h) { return h ? (int64_t)h->last_pruned : 0; }
+
 // The page pool is one allocation sliced into pages (one pool call per join
 // instead of one per page); growing it replaces the allocation.
 // The pool of a single join's result: one block of pages_needed pages (the
@@ -845,7 +847,8 @@ static int self_join_impl(sj_handle h, int64_t item_begin, int64_t item_end, sj_
     out->pair_pages = ri->pair_pages.data();
     out->dist_pages = dist ? ri->dist_pages.data() : nullptr;
     out->n_candidates = h->n_candidates;
-    out->n_evaluated = h->n_evaluated - (int64_t)h->last_pruned;
+    // (the FP64 tile reports what is scheduled, see the header)
+    out->n_evaluated = h->n_evaluated - (h->kernel == SJ_KERNEL_FILTER_F32 ? (int64_t)h->last_pruned : 0);
     out->n_rechecked = (int64_t)rechecked;
     out->reruns = reruns;
     out->kernel = h->kernel;

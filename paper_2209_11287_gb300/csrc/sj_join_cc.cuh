@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join
             if constexpr (PRUNE) {
                 while (v0 < C && cnt < (uint32_t)SLOTS) {
                     const uint32_t out = cc_gather<T, DP, TC, EMIT, RUNS>(W, P, R.r2, C, v0, lane, run, head, cnt);
-                    if constexpr (std::is_same<T, float>::value) pruned += (unsigned long long)out * (unsigned long long)Q;
+                    pruned += (unsigned long long)out * (unsigned long long)Q;
                     v0 += 64u;
                 }
                 if (cnt == 0) break;
