@@ -1098,8 +1098,10 @@ __global__ void k_denum(DenseEnum e, const unsigned long long* __restrict__ off6
 // (6,572 of 1.77 M keys occupied, 243 offsets, count and fill pass) 580 us,
 // now 142; 100,000 of it 469 / 74; 19 cells of 64-D 120 / 29; with every key
 // occupied and 27 offsets (2 M and 1 M x 4-D) as before, 50 / 51 and 209 / 198.
-// Lanes first load the keys of 32 cells and decode their coordinates; the
-// occupied ones are then done one after another.  A block runs over many keys,
+// Lanes first load the keys of `group` cells (32, fewer in a key space that
+// would not give every warp 32) and decode their coordinates; the occupied ones
+// are then done one after another.  (1,500 x 4-D points, a few hundred keys, us:
+// a thread a cell 12.3, 32 cells a warp 19.3, so 5.5; 6-D 108 / 53 / 8.6.)  A block runs over many keys,
 // so the totals take five atomics a block (one address each for the whole
 // grid: 200,000 of them cost more than the runs where every key is occupied).
 // The offsets are the same as k_denum's, in the same order.  (m <= 3: at most 9
@@ -1109,7 +1111,7 @@ template <int MODE>
 __global__ void __launch_bounds__(32 * kDenumWarps) k_denum_warp(DenseEnum e, const unsigned long long* __restrict__ off64,
                                                                  uint32_t* run_cnt, const uint32_t* __restrict__ run_off,
                                                                  Run* runs, Item* items, DenseTotals* tot,
-                                                                 uint32_t slots) {
+                                                                 uint32_t slots, int group) {
     constexpr bool FILL = MODE >= 1;
     constexpr bool COUNT = MODE != 1;
     __shared__ int32_t s_delta[243];  // per offset vector: the key difference,
@@ -1136,11 +1138,11 @@ __global__ void __launch_bounds__(32 * kDenumWarps) k_denum_warp(DenseEnum e, co
     __syncthreads();
     unsigned long long my_eval = 0, my_sq = 0, my_skip = 0, my_cells = 0, my_runs = 0;
     const int64_t warps = (int64_t)gridDim.x * kDenumWarps;
-    for (int64_t k0 = (blockIdx.x * (int64_t)kDenumWarps + (threadIdx.x >> 5)) * 32; k0 < e.K; k0 += warps * 32) {
+    for (int64_t k0 = (blockIdx.x * (int64_t)kDenumWarps + (threadIdx.x >> 5)) * group; k0 < e.K; k0 += warps * group) {
         const int64_t key = k0 + lane;
         unsigned long long a0 = 0;
         uint32_t q = 0;
-        if (key < e.K) {
+        if (lane < group && key < e.K) {
             a0 = off64[key];
             q = (uint32_t)(off64[key + 1] >> 32) - (uint32_t)(a0 >> 32);
             if (MODE == 0 && q == 0) run_cnt[key] = 0;
@@ -1277,9 +1279,12 @@ static void launch_denum(const DenseEnum& e, int device, const unsigned long lon
                          const uint32_t* run_off, Run* runs, Item* items, DenseTotals* tot, uint32_t slots,
                          cudaStream_t s) {
     if (e.m >= 4) {
-        const int64_t groups = (e.K + 32 * kDenumWarps - 1) / (32 * kDenumWarps);
-        const unsigned blocks = (unsigned)std::min<int64_t>(groups, (int64_t)device_sm_count(device) * 12);
-        k_denum_warp<MODE><<<blocks, 32 * kDenumWarps, 0, s>>>(e, off64, run_cnt, run_off, runs, items, tot, slots);
+        const int64_t most = (int64_t)device_sm_count(device) * 12;
+        int group = 32;
+        while (group > 1 && e.K <= most * kDenumWarps * (group / 2)) group >>= 1;
+        const int64_t groups = (e.K + group * kDenumWarps - 1) / (group * kDenumWarps);
+        const unsigned blocks = (unsigned)std::min<int64_t>(groups, most);
+        k_denum_warp<MODE><<<blocks, 32 * kDenumWarps, 0, s>>>(e, off64, run_cnt, run_off, runs, items, tot, slots, group);
     } else {
         k_denum<MODE><<<(unsigned)((e.K + 127) / 128), 128, 0, s>>>(e, off64, run_cnt, run_off, runs, items, tot, slots);
     }
