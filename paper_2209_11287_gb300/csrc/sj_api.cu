@@ -586,6 +586,7 @@ static int run_join(sj_index* ix, ResultImpl* ri, int64_t page_pairs, bool dist,
     jo.band_cap = band_cap;
     jo.dbg = dbg;
     jo.dbg_cap = dbg_cap;
+    jo.share = all_items > 0 ? (double)std::max<int64_t>(item_end - item_begin, 0) / (double)all_items : 1.0;
     int st = SJ_OK;
     if (!ix->ev_tile[0]) {
         SJ_CK(cudaEventCreate(&ix->ev_tile[0]));
@@ -699,6 +700,7 @@ int sj_self_join_to_host(sj_handle h, int32_t* host_pairs, int64_t host_capacity
         jo.capacity = (unsigned long long)device_pairs;
         jo.band = band;
         jo.band_cap = band_cap;
+        jo.share = (double)(i1 - i0) / (double)n_items;
         ix->n_items = i1;  // the kernels stop at the range's end
         if (ix->kernel == SJ_KERNEL_FP64_DMMA)
             st = launch_join_dmma(ix, jo, 0);

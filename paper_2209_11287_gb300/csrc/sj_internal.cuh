@@ -257,6 +257,7 @@ struct JoinOut {
     const void* batch = nullptr;   // device BatchJoin of a batched join, or null
     int4* dbg = nullptr;           // filter dump (sj_debug_filter_dump), or null
     unsigned long long dbg_cap = 0;
+    double share = 1.0;            // part of the index's items that this join is over
 };
 int launch_join_cc(Index* ix, const JoinOut& out, int emit_dist);
 // The small-d FP32 filter without distances (sj_join_f32s.cu).

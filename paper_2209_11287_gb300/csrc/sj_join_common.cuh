@@ -78,8 +78,9 @@ __device__ __forceinline__ void dbg_record_pruned(const JoinParams& P, int32_t q
 // for no work item, for all, or for those of few queries (the others listed in
 // p.big_items), and its launch.
 enum class SparseUse { none, all, few_queries };
-SparseUse f32r_use(const Index* ix, const JoinParams& p);
-int launch_join_f32r(Index* ix, const JoinParams& p);
+// `share`: the part of the index's items that the join is over.
+SparseUse f32r_use(const Index* ix, const JoinParams& p, double share);
+int launch_join_f32r(Index* ix, const JoinParams& p, double share);
 
 JoinParams make_join_params(Index* ix, const JoinOut& out, int emit_dist);
 

@@ -23,7 +23,7 @@ namespace sj {
 
 namespace {
 
-constexpr int kF32rItems = 8;     // items a warp takes at a time
+constexpr int kF32rItems = 8;     // most items a warp takes at a time
 constexpr int kF32rQ = 3;         // most queries of an item dealt with here when there is a list for the others
 constexpr int kF32rRuns = 256;    // runs of a group of them (an item has at most kMaxRuns)
 constexpr int kF32rStage = 256;
@@ -43,8 +43,9 @@ struct F32rWarp {
     int2 stage[kF32rStage];
 };
 
+// take: items a warp takes at a time (8, fewer where all warps would not get as many).
 template <int DP>
-__global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P) {
+__global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P, int take) {
     __shared__ F32rWarp smem[kF32rWarps];
     const float* __restrict__ Y = static_cast<const float*>(P.y);
     const float* __restrict__ H = static_cast<const float*>(P.h);
@@ -57,13 +58,13 @@ __global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P) {
     }
     for (;;) {
         long long first = 0;
-        if (lane == 0) first = (long long)atomicAdd(&P.counters[0], (unsigned long long)kF32rItems);
+        if (lane == 0) first = (long long)atomicAdd(&P.counters[0], (unsigned long long)take);
         first = __shfl_sync(0xffffffffu, first, 0);
         if (first >= P.n_items) break;
         Item I{0, 0, 0, 0};
-        if (lane < kF32rItems && first + lane < P.n_items) I = P.items[first + lane];
+        if (lane < take && first + lane < P.n_items) I = P.items[first + lane];
         if (!SJ_BOUND(P, I.q0 >= 0 && I.q1 <= P.n_points && I.r1 - I.r0 <= kF32rRuns, 51)) I = Item{0, 0, 0, 0};
-        const int have = (int)min((long long)kF32rItems, P.n_items - first);
+        const int have = (int)min((long long)take, P.n_items - first);
         if (P.big_items) {  // items of many queries are left to k_join_f32s
             const bool big = I.q1 - I.q0 > kF32rQ;
             const unsigned m = __ballot_sync(0xffffffffu, big);
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P) {
 }
 
 template <int DP>
-int launch_f32r_d(Index* ix, const JoinParams& p) {
+int launch_f32r_d(Index* ix, const JoinParams& p, double items) {
     auto kern = k_join_f32r<DP>;
     static std::atomic<int> cached{0};  // resident CTAs per SM (a property of the kernel)
     int per_sm = cached.load(std::memory_order_relaxed);
@@ -209,9 +210,12 @@ int launch_f32r_d(Index* ix, const JoinParams& p) {
         if (per_sm < 1) per_sm = 1;
         cached.store(per_sm, std::memory_order_relaxed);
     }
-    const long long need = (ix->n_items + kF32rItems * kF32rWarps - 1) / (kF32rItems * kF32rWarps);
-    const long long blocks = std::max<long long>(1, std::min<long long>(need, (long long)device_sm_count(ix->device) * per_sm));
-    kern<<<(unsigned)blocks, 32 * kF32rWarps, 0, ix->stream>>>(p);
+    const long long most = (long long)device_sm_count(ix->device) * per_sm;
+    int take = 1;  // (4-D 3,000 points, 31 evaluations an item: 8 at a time 20.9 us, 1 12.5)
+    while (take < kF32rItems && items > (double)(most * kF32rWarps * take)) take <<= 1;
+    const double need = items / (take * kF32rWarps) + 1.0;
+    const long long blocks = need < (double)most ? (long long)need : most;
+    kern<<<(unsigned)blocks, 32 * kF32rWarps, 0, ix->stream>>>(p, take);
     note_launch();
     SJ_CK(cudaGetLastError());
     return SJ_OK;
@@ -219,33 +223,43 @@ int launch_f32r_d(Index* ix, const JoinParams& p) {
 
 }  // namespace
 
-// Taken for single joins whose cells are sparse.  Evenly filled cells (a point's
-// own cell holds at most 1.6 times the mean cell): for all items below 2.5
-// queries an item (1.9 for padded d = 8, whose candidates cost more to load) and
-// 160 (300) evaluations an item.  Both kernels, us, by queries an item: uniform
-// 4-D 1.1 754 / 155, 1.4 667 / 274, 2.0 540 / 352, 3.2 419 / 475; 3-D 1.6 283 /
-// 88, 3.9 156 / 151; 2-D 1.8 375 / 164, 2.8 286 / 210, 5.1 195 / 279; 5-D 1.8
-// 323 / 245, 3.8 266 / 500; 6-D 1.2 336 / 189, 1.8 348 / 382.  Crowded and single
-// cells side by side: for the items of up to 3 queries, below 3.2 queries an item
-// as n / (cells + n / 16) counts them (clusters over noise, k_join_f32s alone / k_join_f32r alone / shared: 3-D 1.6
-// 467 / 333 / 315, 2.7 389 / 927 / 346, 4-D 2.3 596 / - / 485, 2-D 3.2 337 / 488 /
-// 293, 4.7 154 / - / 166; at 2 and 4 queries 347 and 362 for the 3-D 2.7; shared
-// on even cells it costs the second launch: uniform 4-D 1.4 305).  (Batched joins
-// and the filter's recording mode keep k_join_f32s.)
-SparseUse f32r_use(const Index* ix, const JoinParams& p) {
+// Taken for single joins whose cells are sparse, by the queries q and the
+// evaluations e of an item and the number of items, counted as cells + n / 16
+// (the part of them that a range of items is).  The lines were fitted to 545
+// states (uniform and clustered, 2-D to 8-D, 1 to 40 neighbours, 300 to 1,000,000
+// points) so that none is slower than k_join_f32s by more than 4%; tile us,
+// k_join_f32s / this kernel alone / shared.
+// Evenly filled cells (a point's own cell holds at most 1.4 times the mean
+// cell), this kernel alone.  Padded d <= 4: q < 2.5, and e < 160 from 2^16 items
+// on (uniform 4-D 1,000,000 points: q 1.3 677 / 267, q 1.7, e 102 551 / 349, q
+// 2.3, e 207 460 / 423; 3-D 300,000, q 4.1 89 / 142), else e < 60 (4-D 3,000, e 31
+// 14.8 / 12.5; 1,000, e 85 13.2 / 14.5).  Padded d = 8: q < 1.9, and e < 250 from
+// 2^17 items on (5-D 1,000,000: e 99 1187 / 639; 6-D, q 1.8, e 732 1771 / 1947),
+// else e < 60 (6-D 10,000: e 77 29 / 24, e 185 34 / 41).
+// Other cells, the items of up to 3 queries, where there are enough of them for
+// two launches: 2^17 items, q < 2.5, e < 400 (clusters over noise, 3-D 342,000
+// items 520 / 1120 / 472, 4-D 511,000 588 / 606 / 432, 134,000 183 / 330 / 180,
+// 49,000 76 / 162 / 93, 3-D 811 17 / 25 / 28).  (Batched joins and the filter's
+// recording mode keep k_join_f32s.)
+static double f32r_items(const Index* ix, double share) { return ((double)ix->n_cells + (double)ix->n / kQMax) * share; }
+
+SparseUse f32r_use(const Index* ix, const JoinParams& p, double share) {
     if (p.batch || p.dbg || ix->n_cells <= 0) return SparseUse::none;
-    const double n = (double)ix->n, cells = (double)ix->n_cells, items = cells + n / kQMax;
-    if ((double)ix->sum_sq / n > 1.6 * n / cells) return n < 3.2 * items ? SparseUse::few_queries : SparseUse::none;
-    const bool small = ix->dp <= 4;
-    return n < (small ? 2.5 : 1.9) * items && (double)ix->n_evaluated < (small ? 160.0 : 300.0) * items ? SparseUse::all
-                                                                                               : SparseUse::none;
+    const double n = (double)ix->n, cells = (double)ix->n_cells, items = f32r_items(ix, share);
+    const double q = n / f32r_items(ix, 1.0), e = (double)ix->n_evaluated / f32r_items(ix, 1.0);
+    if ((double)ix->sum_sq / n > 1.4 * n / cells)
+        return items >= (1 << 17) && q < 2.5 && e < 400.0 ? SparseUse::few_queries : SparseUse::none;
+    const bool take = ix->dp <= 4 ? q < 2.5 && e < (items >= (1 << 16) ? 160.0 : 60.0)
+                                  : q < 1.9 && e < (items >= (1 << 17) ? 250.0 : 60.0);
+    return take ? SparseUse::all : SparseUse::none;
 }
 
-int launch_join_f32r(Index* ix, const JoinParams& p) {
+int launch_join_f32r(Index* ix, const JoinParams& p, double share) {
+    const double items = f32r_items(ix, share);
     switch (ix->dp) {
-        case 2: return launch_f32r_d<2>(ix, p);
-        case 4: return launch_f32r_d<4>(ix, p);
-        case 8: return launch_f32r_d<8>(ix, p);
+        case 2: return launch_f32r_d<2>(ix, p, items);
+        case 4: return launch_f32r_d<4>(ix, p, items);
+        case 8: return launch_f32r_d<8>(ix, p, items);
         default:
             set_error("no small-d FP32 kernel for padded dimension %d", ix->dp);
             return SJ_ERR_UNSUPPORTED;

@@ -611,7 +611,7 @@ bool f32s_supported(const Index* ix, int emit_dist) {
 int launch_join_f32s(Index* ix, const JoinOut& out) {
     JoinParams p = make_join_params(ix, out, 0);
     Scratch tmp(ix->stream);  // (released after the launches that use it, stream-ordered)
-    SparseUse sparse = f32r_use(ix, p);
+    SparseUse sparse = f32r_use(ix, p, out.share);
     if (sparse == SparseUse::few_queries) {
         const int st = tmp.alloc(&p.big_items, (size_t)ix->n_items);
         if (st == SJ_ERR_OOM) {  // no room for the list: k_join_f32s takes all items
@@ -622,7 +622,7 @@ int launch_join_f32s(Index* ix, const JoinOut& out) {
             return st;
         }
     }
-    if (sparse != SparseUse::none) SJ_TRY(launch_join_f32r(ix, p));
+    if (sparse != SparseUse::none) SJ_TRY(launch_join_f32r(ix, p, out.share));
     if (sparse == SparseUse::all) return SJ_OK;
     switch (ix->dp) {
         case 2: return launch_f32s_d<2>(ix, p);

@@ -156,12 +156,13 @@ def test_list_of_the_items_of_many_queries():
     """Crowded cells among single points: without the list that the two FP32
     filters share the items by, one of them takes all."""
     g = np.random.Generator(np.random.PCG64(5))
-    x = g.random((7001, 3))
-    x[:2300] = 0.5 + 0.02 * (g.random((2300, 3)) - 0.5) + 0.25 * g.integers(0, 2, (2300, 1))
-    eps = (0.3 / 7001) ** (1.0 / 3)
+    n = 260_000
+    x = g.random((n, 3))
+    eps = (0.3 / n) ** (1.0 / 3)
+    x[: n // 4] = x[g.integers(n // 2, n // 2 + 4000, n // 4)] + 0.05 * eps * g.random((n // 4, 3))
     ref = oracle.join(x, eps)
     h = binding.sj_build_index(torch.from_numpy(x).cuda(), eps,
-                               binding.sj_default_options(kernel="filter_f32", max_pairs_hint=1 << 22))
+                               binding.sj_default_options(kernel="filter_f32", max_pairs_hint=1 << 24))
 
     def run():
         launches = binding.sj_kernel_launches()

@@ -43,11 +43,11 @@ SCRIPT = textwrap.dedent("""
     g = np.random.Generator(np.random.PCG64(11))
     for d in (2, 3, 4, 6, 8):
         for crowded in (False, True):
-            n = 6001
+            n = 6001 if not crowded else 260_000 if d < 6 else 30_000
             x = g.random((n, d))
             eps = (0.3 / n) ** (1.0 / d)
-            if crowded:  # a third of the points in a few cells
-                x[: n // 3] = 0.5 + 0.02 * eps * (g.random((n // 3, d)) - 0.5) + eps * g.integers(0, 40, (n // 3, 1))
+            if crowded:  # a quarter of the points close to a few others
+                x[: n // 4] = x[g.integers(n // 2, n // 2 + n // 64, n // 4)] + 0.05 * eps * g.random((n // 4, d))
             ref = oracle.join(x, eps)
             for sym in (1, 0):
                 h = binding.sj_build_index(torch.from_numpy(x).cuda(), eps,
