@@ -548,7 +548,7 @@ SJ_API int sj_dbscan(const sj_result* r, int64_t n, int32_t min_pts, int32_t* la
  * dist_out n x k (row-major; -1 and +inf past the found ones), found_out n
  * (neighbours found, at most k: fewer when the point has fewer than k other
  * points within eps); host or device memory.  Takes 20 bytes of scratch a
- * pair, 12 where that finds no room.  Synchronous.  Errors:
+ * pair, 12 where that finds no room and for many long neighbourhoods.  Synchronous.  Errors:
  * SJ_ERR_ARG (no distances, a batched result, k outside 1 .. 1024),
  * SJ_ERR_RESULT_OVERFLOW, SJ_ERR_OOM, SJ_ERR_CUDA.
  */

@@ -79,16 +79,20 @@ struct __align__(16) KnnEntry {
 // kNN from a join: bucket sizes (self pairs left out) and every pair's place
 // in its bucket, so the bucketing below needs no second atomic per pair (9.4 M
 // pairs, both kernels: 213 us with an atomic in each and two stores per pair,
-// 185 us so) ...  These take 20 bytes a pair; where that finds no room, the
-// entries are split (12 bytes a pair: place null, one atomic more).
+// 185 us so) ...  These take 20 bytes a pair; where that finds no room, or
+// where it is far more than L2 holds and the buckets are long (knn_split), the
+// entries are split (12 bytes a pair: no place, one atomic more).
+template <bool PLACE>
 __global__ void k_knn_degree(const int2* __restrict__ pairs, long long count, uint32_t* deg,
                              uint32_t* __restrict__ place) {
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < count;
          p += (long long)gridDim.x * blockDim.x) {
         const int2 e = pairs[p];
         if (e.x == e.y) continue;
-        const uint32_t at = atomicAdd(&deg[e.x], 1u);
-        if (place) place[p] = at;
+        if constexpr (PLACE)
+            place[p] = atomicAdd(&deg[e.x], 1u);
+        else
+            atomicAdd(&deg[e.x], 1u);
     }
 }
 
@@ -116,6 +120,17 @@ __global__ void k_knn_bucket_split(const int2* __restrict__ pairs, const double*
         nb_dist[s] = dist[p];
     }
 }
+
+// Long buckets beyond L2 fill their lines before they are evicted only if few of
+// them are open at a time: then the fewer bytes of the split entries count for
+// more than the second atomic, most of all where the pairs of a point lie
+// scattered in the list (a tensor-core filter's).  The whole call at k = 8, whole
+// / split, us: 30,000 points x 1,700 neighbours 16-D clusters 2295 / 1696, 1,780
+// uniform 16-D 2522 / 1867, 1,370 3-D 1494 / 1468; 100,000 x 770 16-D 3873 / 2942,
+// x 640 3-D 2238 / 1983, x 300 16-D clusters 1407 / 1241, x 285 3-D 1013 / 974, x
+// 146 541 / 527; 30,000 x 630 706 / 727; shorter or fewer: 1,000,000 x 41 1849 /
+// 1919, 30,000 x 360 432 / 460.
+static bool knn_split(long long count, int64_t n) { return count >= (3 << 22) && count / n >= 128; }
 
 // Where the selection reads its entries (as KnnEntry's four words).
 struct KnnWhole {
@@ -174,14 +189,13 @@ __global__ void __launch_bounds__(32 * kKnnWarps) k_knn_select(int64_t n, int k,
         const int full = min(kKnnList - 31, max(64, 2 * k));  // cut back from this many on
         int m = 0;
         KnnKey bar{0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};  // the k-th smallest so far
+        int4 next = make_int4(0, 0, 0, 0);  // (a chunk ahead: its load does not wait for the list)
+        if (a + (uint32_t)lane < b) next = src[a + (uint32_t)lane];
         for (uint32_t s0 = a; s0 < b; s0 += 32) {
             const uint32_t s = s0 + (uint32_t)lane;
-            int4 e = make_int4(0, 0, 0, 0);
-            bool in = false;
-            if (s < b) {
-                e = src[s];
-                in = knn_minus_lt(0, knn_key(e), bar) != 0;
-            }
+            const int4 e = next;
+            if (b - s0 > 32u + (uint32_t)lane) next = src[s + 32u];
+            const bool in = s < b && knn_minus_lt(0, knn_key(e), bar) != 0;
             const unsigned w = __ballot_sync(0xffffffffu, in);
             if (in) list[m + __popc(w & ((1u << lane) - 1u))] = e;
             m += __popc(w);
@@ -314,7 +328,7 @@ extern "C" int sj_knn_from_join(const sj_result* r, int64_t n, int32_t k, int32_
     SJ_TRY(tmp.alloc(&oi, (size_t)n * k));
     SJ_TRY(tmp.alloc(&od, (size_t)n * k));
     SJ_TRY(tmp.alloc(&of, (size_t)n));
-    int st = dev_alloc_t(&nb, slots, s);
+    int st = knn_split(count, n) ? SJ_ERR_OOM : dev_alloc_t(&nb, slots, s);
     if (st == SJ_OK) st = dev_alloc_t(&place, slots, s);
     if (st == SJ_ERR_OOM) {  // the split entries then
         clear_error();
@@ -331,7 +345,10 @@ extern "C" int sj_knn_from_join(const sj_result* r, int64_t n, int32_t k, int32_
     }
     SJ_CK(cudaMemsetAsync(deg, 0, (size_t)n * sizeof(uint32_t), s));
     if (count > 0) {
-        k_knn_degree<<<grid_for(count, dev), 256, 0, s>>>(pairs, count, deg, place);
+        if (place)
+            k_knn_degree<true><<<grid_for(count, dev), 256, 0, s>>>(pairs, count, deg, place);
+        else
+            k_knn_degree<false><<<grid_for(count, dev), 256, 0, s>>>(pairs, count, deg, nullptr);
         note_launch();
         SJ_CK(cudaGetLastError());
     }
