@@ -135,7 +135,7 @@ struct TcSmem {
     uint8_t rfl[kMaxRuns];
 };
 
-// Operand stages: as many as fit (up to 6) in the 227 KB of shared memory a
+// Operand stages: as many as fit (up to 8) in the 227 KB of shared memory a
 // CTA may use next to the query tile and the rest.
 constexpr size_t kSmemMax = 232448;
 template <int KP>
