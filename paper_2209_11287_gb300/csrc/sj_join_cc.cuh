@@ -61,6 +61,7 @@ struct CcWarpSmem {
     int32_t ring_j[PRUNE ? RING : 1];
     uint8_t ring_f[PRUNE ? RING : 1];
     float blo[PRUNE ? DP : 1], bhi[PRUNE ? DP : 1];
+    unsigned long long pruned;  // evaluations that the prune removed (lane 0; not in a register: FP64 has none to spare)
 };
 
 // Compaction step of the prune, d <= 8: candidates [v0, v0 + 64) of the item,
@@ -305,7 +306,8 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join
     ItemSmem<T, DP, RUNS>& S = W.it;
     WarpStage st{W.stage, EMIT ? W.sdist : nullptr, 0, 0};
     BandQ bq{0, 0};
-    unsigned long long rechecked = 0, pruned = 0;  // (pruned: the same in all lanes)
+    unsigned long long rechecked = 0;
+    if (PRUNE && lane == 0) W.pruned = 0;
 
     long long next = 0;
     if (lane == 0) next = (long long)atomicAdd(&P.counters[0], 1ull);
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join
             if constexpr (PRUNE) {
                 while (v0 < C && cnt < (uint32_t)SLOTS) {
                     const uint32_t out = cc_gather<T, DP, TC, EMIT, RUNS>(W, P, R.r2, C, v0, lane, run, head, cnt);
-                    pruned += (unsigned long long)out * (unsigned long long)Q;
+                    if (lane == 0) W.pruned += (unsigned long long)(out * (uint32_t)Q);
                     v0 += 64u;
                 }
                 if (cnt == 0) break;
@@ -542,7 +544,7 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join
     }
     band_q_close(bq, P, lane);
     stage_flush(st, P, lane);
-    if (lane == 0 && pruned) atomicAdd(&P.counters[6], pruned);
+    if (PRUNE && lane == 0 && W.pruned) atomicAdd(&P.counters[6], W.pruned);
     for (int o = 16; o > 0; o >>= 1) rechecked += __shfl_down_sync(0xffffffffu, rechecked, o);
     if (lane == 0 && rechecked) atomicAdd(&P.counters[2], rechecked);
 }

@@ -261,6 +261,7 @@ constexpr int kTcChunk = 64;
 struct TcRecords {
     unsigned long long base;  // next reserved record
     int left;                 // reserved records left (warp-uniform)
+    bool over;                // the reservation goes past the queue
 };
 
 // Squared distance of two kernel-coordinate rows in binary32, rows of dp floats
@@ -381,10 +382,11 @@ __device__ __forceinline__ void tc_record(TcRecords& rec, const JoinParams& P, i
         const int used = n - rec.left;
         rec.base = fresh + (unsigned long long)used;
         rec.left = kTcChunk - used;
+        rec.over = fresh + kTcChunk > P.band_cap >> 1;
     }
-    const unsigned long long room = P.band_cap >> 1;
-    if (e.x != 0 && pos < room) reinterpret_cast<int4*>(P.band)[pos] = e;
-    if (rec.base > room) tc_resolve_here(P, lane, pos < room ? make_int4(0, 0, 0, 0) : e);  // (uniform)
+    const bool fits = pos < P.band_cap >> 1;
+    if (e.x != 0 && fits) reinterpret_cast<int4*>(P.band)[pos] = e;
+    if (rec.over) tc_resolve_here(P, lane, fits ? make_int4(0, 0, 0, 0) : e);  // (uniform)
 }
 
 // DBG: the recording instantiation of the filter dump (a test aid; the join
@@ -756,7 +758,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_join_tc(JoinParams P, TcParam
         const int quarter = warp & 3;  // TMEM lanes 32 quarter .. + 31
         const int part = ew >> 2;      // 32-column chunks part, part + EPI / 4, ...
         constexpr int CSTEP = 32 * (SM::EPI / 4);
-        TcRecords rec{0, 0};
+        TcRecords rec{0, 0, false};
         uint32_t it_i = 0, it_ph = 0, acc = 0, acc_ph = 0;
         for (;;) {
             if (!bar_wait_warp(&S.item_full[it_i], it_ph, abort)) break;

@@ -51,6 +51,27 @@ __device__ __forceinline__ float refine_sq(const float* __restrict__ a, const fl
     return s;
 }
 
+// Pairs of several batched instances in a warp: a reservation for each instance,
+// its lanes one after another.  (Out of line: rare, and the kernel's registers
+// are few: 2M x 4-D 670 us with it inlined three times, 634 so.)
+__device__ __noinline__ void resolve_emit_mixed(const JoinParams& P, int lane, int gid, int nout, int32_t qid, int32_t cid,
+                                                double dist) {
+    const BatchJoin& B = *P.batch;
+    const unsigned same = __match_any_sync(0xffffffffu, nout > 0 ? gid : -1);
+    const unsigned two = __ballot_sync(0xffffffffu, nout == 2), lt = (1u << lane) - 1u;
+    const int first = __ffs(same) - 1;
+    unsigned long long at = 0;
+    if (nout > 0 && lane == first)
+        at = atomicAdd(&B.cursor[gid], (unsigned long long)(__popc(same) + __popc(same & two)));
+    at = __shfl_sync(0xffffffffu, at, first) + (unsigned)(__popc(same & lt) + __popc(same & two & lt));
+    for (int u = 0; u < nout; ++u) {
+        const long long slot = batch_slot(B, gid, at + (unsigned)u);
+        if (slot < 0) continue;
+        B.pool[slot] = u == 0 ? make_int2(qid, cid) : make_int2(cid, qid);
+        if (P.emit_dist) B.dpool[slot] = dist;
+    }
+}
+
 // Bound by the latency of its gathers (positions to ids and rows, cursor and
 // page of a flush), so a pair's first loads do not wait for one another
 // (500,000 x 16-D mixture, build, filter and this kernel: the ids loaded after
@@ -84,18 +105,21 @@ __global__ void __launch_bounds__(32 * kResolveWarps, kResolveBlocks) k_resolve(
             qid = P.perm[qs];
             cid = P.perm[cs];
             const int li = inst_of ? inst_of[qs] : 0;
-            bool in = certain, exact = EMIT && certain;  // (exact: the binary64 sum is needed)
-            if (EMIT || !certain) ++decided;
-            if (!certain) {
-                const float s32 = refine_sq<DP>(Y + (int64_t)qs * DP, Y + (int64_t)cs * DP);
-                const float2 r = inst_of ? P.batch->inst_refine[li] : make_float2(P.refine_out, P.refine_in);
-                in = s32 < r.y;
-                exact = (EMIT || !in) && !(s32 > r.x);
-            }
-            if (exact) {
-                const double s = direct_sq(P.xs + (int64_t)qs * DP, P.xs + (int64_t)cs * DP, P.d);
-                in = s <= (inst_of ? P.batch->inst_e2[li] : P.e2);
-                if (EMIT && in) dist = sqrt(s);
+            bool in = certain;
+            if (EMIT || !certain) {
+                ++decided;
+                bool exact = EMIT;  // (the binary64 sum is needed)
+                if (!certain) {
+                    const float s32 = refine_sq<DP>(Y + (int64_t)qs * DP, Y + (int64_t)cs * DP);
+                    const float2 r = inst_of ? P.batch->inst_refine[li] : make_float2(P.refine_out, P.refine_in);
+                    in = s32 < r.y;
+                    exact = (EMIT || !in) && !(s32 > r.x);
+                }
+                if (exact) {
+                    const double s = direct_sq(P.xs + (int64_t)qs * DP, P.xs + (int64_t)cs * DP, P.d);
+                    in = s <= (inst_of ? P.batch->inst_e2[li] : P.e2);
+                    if (EMIT && in) dist = sqrt(s);
+                }
             }
             if (in) nout = e.y < 0 && cs != qs ? 2 : 1;
             if (inst_of) {
@@ -114,20 +138,7 @@ __global__ void __launch_bounds__(32 * kResolveWarps, kResolveBlocks) k_resolve(
             if (some == 0u) return;
             const int g0 = __shfl_sync(0xffffffffu, gid, __ffs(some) - 1);
             if (!__all_sync(0xffffffffu, nout == 0 || gid == g0)) {
-                const BatchJoin& B = *P.batch;
-                const unsigned same = __match_any_sync(0xffffffffu, nout > 0 ? gid : -1);
-                const unsigned two = __ballot_sync(0xffffffffu, nout == 2), lt = (1u << lane) - 1u;
-                const int first = __ffs(same) - 1;
-                unsigned long long at = 0;
-                if (nout > 0 && lane == first)
-                    at = atomicAdd(&B.cursor[gid], (unsigned long long)(__popc(same) + __popc(same & two)));
-                at = __shfl_sync(0xffffffffu, at, first) + (unsigned)(__popc(same & lt) + __popc(same & two & lt));
-                for (int u = 0; u < nout; ++u) {
-                    const long long slot = batch_slot(B, gid, at + (unsigned)u);
-                    if (slot < 0) continue;
-                    B.pool[slot] = u == 0 ? make_int2(qid, cid) : make_int2(cid, qid);
-                    if (EMIT) B.dpool[slot] = dist;
-                }
+                resolve_emit_mixed(P, lane, gid, nout, qid, cid, dist);
                 __syncwarp();
                 return;
             }
@@ -151,21 +162,23 @@ __global__ void __launch_bounds__(32 * kResolveWarps, kResolveBlocks) k_resolve(
     // 96 joins in one batch: blocks a grid apart 6.52 ms, runs of 4 6.22, 16
     // 6.19, 64 6.17; one join of the 16-D mixture 2.64 / 2.67 / 2.67 / 2.77 ms,
     // long runs leave warps idle.
-    // Few records are spread over all warps in blocks of fewer (a block's pairs
-    // are dealt with 32 at a time, one after another).  4,000 x 64-D points with
+    // With distances few records are spread over all warps in blocks of fewer (a
+    // block's pairs are dealt with 32 at a time, one after another, and each takes
+    // the latency of its binary64 sums).  4,000 x 64-D points with
     // distances, 61,000 pairs, filter and this kernel: 188 us with blocks of 32
     // and every pair in binary32 first, 128 so and with the certain ones in
     // binary64 at once.
     const unsigned long long warps = (unsigned long long)gridDim.x * kResolveWarps;
     int size = 32;  // records of a block
-    while (size > 8 && count < warps * (unsigned)(size / 2)) size >>= 1;
+    if constexpr (EMIT)
+        while (size > 8 && count < warps * (unsigned)(size / 2)) size >>= 1;
     const unsigned long long blocks = (count + (unsigned)size - 1) / (unsigned)size;
     const unsigned long long run = min((unsigned long long)kResolveRun, max(1ull, blocks / (2 * warps)));
     int of_list = -1;  // batch: the instance of the waiting pairs
     unsigned long long r = (unsigned long long)blockIdx.x * kResolveWarps + wid, k_run = 0;
     for (; r * run + k_run < blocks; k_run + 1 < run ? ++k_run : (k_run = 0, r += warps)) {
         const unsigned long long b = (r * run + k_run) * (unsigned)size;
-        const int4 e = lane < size && b + lane < count ? records[b + lane] : make_int4(0, 0, 0, 0);
+        const int4 e = (!EMIT || lane < size) && b + lane < count ? records[b + lane] : make_int4(0, 0, 0, 0);
         if (inst_of) {  // what waits of another instance goes first, so that a warp of pairs has one
             const int cs = (int)((uint32_t)e.w & ~kMirrorBit);
             const unsigned some = __ballot_sync(0xffffffffu, e.x != 0);
