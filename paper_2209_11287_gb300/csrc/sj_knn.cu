@@ -132,17 +132,22 @@ __global__ void k_knn_bucket_split(const int2* __restrict__ pairs, const double*
 // 1919, 30,000 x 360 432 / 460.
 static bool knn_split(long long count, int64_t n) { return count >= (3 << 22) && count / n >= 128; }
 
-// Where the selection reads its entries (as KnnEntry's four words).
+// Where the selection reads its entries (as KnnEntry's four words), and whether
+// it loads a chunk ahead, so that the load does not wait for the list: it pays for
+// long buckets (150 neighbours of 100,000 points 502 / 488 us), not for short ones
+// (47 neighbours 150 / 160).
 struct KnnWhole {
+    static constexpr bool kAhead = false;
     const int4* e;
-    __device__ __forceinline__ int4 operator[](uint32_t s) const { return e[s]; }
+    __device__ __forceinline__ int4 operator[](uint32_t s) const { return __ldg(e + s); }
 };
 struct KnnSplit {
+    static constexpr bool kAhead = true;
     const int32_t* idx;
     const double* dist;
     __device__ __forceinline__ int4 operator[](uint32_t s) const {
-        const long long d = __double_as_longlong(dist[s]);
-        return make_int4((int)d, (int)(d >> 32), idx[s], 0);
+        const long long d = __double_as_longlong(__ldg(dist + s));
+        return make_int4((int)d, (int)(d >> 32), __ldg(idx + s), 0);
     }
 };
 
@@ -189,12 +194,16 @@ __global__ void __launch_bounds__(32 * kKnnWarps) k_knn_select(int64_t n, int k,
         const int full = min(kKnnList - 31, max(64, 2 * k));  // cut back from this many on
         int m = 0;
         KnnKey bar{0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};  // the k-th smallest so far
-        int4 next = make_int4(0, 0, 0, 0);  // (a chunk ahead: its load does not wait for the list)
-        if (a + (uint32_t)lane < b) next = src[a + (uint32_t)lane];
+        int4 next = make_int4(0, 0, 0, 0);
+        if (Src::kAhead && a + (uint32_t)lane < b) next = src[a + (uint32_t)lane];
         for (uint32_t s0 = a; s0 < b; s0 += 32) {
             const uint32_t s = s0 + (uint32_t)lane;
-            const int4 e = next;
-            if (b - s0 > 32u + (uint32_t)lane) next = src[s + 32u];
+            int4 e = next;
+            if constexpr (Src::kAhead) {
+                if (b - s0 > 32u + (uint32_t)lane) next = src[s + 32u];
+            } else if (s < b) {
+                e = src[s];
+            }
             const bool in = s < b && knn_minus_lt(0, knn_key(e), bar) != 0;
             const unsigned w = __ballot_sync(0xffffffffu, in);
             if (in) list[m + __popc(w & ((1u << lane) - 1u))] = e;
