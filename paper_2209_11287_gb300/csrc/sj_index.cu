@@ -1280,8 +1280,8 @@ static void launch_denum(const DenseEnum& e, int device, const unsigned long lon
                          cudaStream_t s) {
     if (e.m >= 4) {
         const int64_t most = (int64_t)device_sm_count(device) * 12;
-        int group = 32;
-        while (group > 1 && e.K <= most * kDenumWarps * (group / 2)) group >>= 1;
+        int group = 32;  // (a third of the blocks: each costs a table and five atomics)
+        while (group > 1 && e.K <= most / 3 * kDenumWarps * (group / 2)) group >>= 1;
         const int64_t groups = (e.K + group * kDenumWarps - 1) / (group * kDenumWarps);
         const unsigned blocks = (unsigned)std::min<int64_t>(groups, most);
         k_denum_warp<MODE><<<blocks, 32 * kDenumWarps, 0, s>>>(e, off64, run_cnt, run_off, runs, items, tot, slots, group);

@@ -552,9 +552,11 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join
 // Whether a join's candidates pass the bounding-box prune: where items have more
 // than 140 candidates, so that it saves whole chunks (of 128 candidates in FP64,
 // 64 in FP32) and not slots of one, and in FP64 more than 300 evaluations, for
-// its own cost an item.  Planar cells keep 83% of their candidates, so padded
-// d = 2 goes without it, and so do joins without an index (the box of 16
-// arbitrary points spans everything) and batches (no radius per instance for the
+// its own cost an item; in FP64 with few items, which leave the chip waiting for
+// single ones, above 90 (30,000 x 3-D, 97 candidates: 67.8 / 63.8).  Planar cells
+// keep 83% of their candidates, so padded d = 2 goes without it in FP64 and above
+// 70 candidates with it in FP32; joins without an index go without (the box of 16
+// arbitrary points spans everything), and batches (no radius per instance for the
 // FP64 tile).  Tile times without / with it, us, by candidates an item (200,000
 // points): FP64 3-D 75 196 / 233, 150 362 / 273, 718 1183 / 1000; 4-D 24 252 /
 // 325, 94 219 / 271, 175 337 / 267, 644 1028 / 717; 6-D 50 572 / 788, 149 (200
@@ -563,11 +565,13 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join
 // index 6468 / 7373.  FP64 with distances 4-D 24 263 / 412, 175 335 / 289.  FP32
 // with distances 3-D 39 91 / 102, 75 103 / 104, 150 150 / 144; 4-D 24 115 / 153,
 // 94 99 / 106, 175 102 / 99, 644 204 / 176; 6-D 50 296 / 334, 149 474 / 428,
-// 2026 766 / 565; 2-D 10 83 / 91, 76 206 / 197.
+// 2026 766 / 565; 2-D 10 83 / 91, 37 115 / 115, 76 206 / 197, clusters 74 245 / 231.
 inline bool cc_prune(const Index* ix, const JoinParams& p, bool fp64) {
-    if (p.batch || ix->m == 0 || ix->n_cells <= 0 || ix->dp == 2) return false;
-    const double n = (double)ix->n, ev = (double)ix->n_evaluated;
-    return ev > 140.0 * n && (!fp64 || ev > 300.0 * ((double)ix->n_cells + n / kQMax));
+    if (p.batch || ix->m == 0 || ix->n_cells <= 0) return false;
+    const double n = (double)ix->n, ev = (double)ix->n_evaluated, items = (double)ix->n_cells + n / kQMax;
+    if (ix->dp == 2) return !fp64 && ev > 70.0 * n;
+    if (fp64 && items < 8192.0) return ev > 90.0 * n && ev > 300.0 * items;
+    return ev > 140.0 * n && (!fp64 || ev > 300.0 * items);
 }
 
 template <typename T, int DP, bool EMIT, int RUNS, bool PRUNE>
@@ -594,7 +598,7 @@ inline int launch_dper(Index* ix, const JoinParams& p) {
 template <typename T, int DP, bool EMIT>
 inline int launch_dpe(Index* ix, const JoinParams& p) {
     if constexpr (DP <= 8) {
-        if constexpr (DP > 2)
+        if constexpr (DP > 2 || std::is_same<T, float>::value)
             if (cc_prune(ix, p, std::is_same<T, double>::value))
                 return ix->m <= 4 ? launch_dper<T, DP, EMIT, 28, true>(ix, p)
                                   : launch_dper<T, DP, EMIT, kMaxRuns, true>(ix, p);

@@ -43,9 +43,10 @@ struct F32rWarp {
     int2 stage[kF32rStage];
 };
 
-// take: items a warp takes at a time (8, fewer where all warps would not get as many).
-template <int DP>
-__global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P, int take) {
+// TAKE: items a warp takes at a time (8, fewer where all warps would not get as
+// many; a run-time number spilled for padded d = 8: 1,000,000 x 5-D 811 / 851 us).
+template <int DP, int TAKE>
+__global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P) {
     __shared__ F32rWarp smem[kF32rWarps];
     const float* __restrict__ Y = static_cast<const float*>(P.y);
     const float* __restrict__ H = static_cast<const float*>(P.h);
@@ -58,13 +59,13 @@ __global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P, int
     }
     for (;;) {
         long long first = 0;
-        if (lane == 0) first = (long long)atomicAdd(&P.counters[0], (unsigned long long)take);
+        if (lane == 0) first = (long long)atomicAdd(&P.counters[0], (unsigned long long)TAKE);
         first = __shfl_sync(0xffffffffu, first, 0);
         if (first >= P.n_items) break;
+        const int have = (int)min((long long)TAKE, P.n_items - first);
         Item I{0, 0, 0, 0};
-        if (lane < take && first + lane < P.n_items) I = P.items[first + lane];
+        if (lane < have) I = P.items[first + lane];
         if (!SJ_BOUND(P, I.q0 >= 0 && I.q1 <= P.n_points && I.r1 - I.r0 <= kF32rRuns, 51)) I = Item{0, 0, 0, 0};
-        const int have = (int)min((long long)take, P.n_items - first);
         if (P.big_items) {  // items of many queries are left to k_join_f32s
             const bool big = I.q1 - I.q0 > kF32rQ;
             const unsigned m = __ballot_sync(0xffffffffu, big);
@@ -200,9 +201,9 @@ __global__ void __launch_bounds__(32 * kF32rWarps) k_join_f32r(JoinParams P, int
     if (lane == 0 && W.rechecked) atomicAdd(&P.counters[2], W.rechecked);
 }
 
-template <int DP>
-int launch_f32r_d(Index* ix, const JoinParams& p, double items) {
-    auto kern = k_join_f32r<DP>;
+template <int DP, int TAKE>
+int launch_f32r_dt(Index* ix, const JoinParams& p, double items) {
+    auto kern = k_join_f32r<DP, TAKE>;
     static std::atomic<int> cached{0};  // resident CTAs per SM (a property of the kernel)
     int per_sm = cached.load(std::memory_order_relaxed);
     if (per_sm == 0) {
@@ -210,15 +211,25 @@ int launch_f32r_d(Index* ix, const JoinParams& p, double items) {
         if (per_sm < 1) per_sm = 1;
         cached.store(per_sm, std::memory_order_relaxed);
     }
-    const long long most = (long long)device_sm_count(ix->device) * per_sm;
-    int take = 1;  // (4-D 3,000 points, 31 evaluations an item: 8 at a time 20.9 us, 1 12.5)
-    while (take < kF32rItems && items > (double)(most * kF32rWarps * take)) take <<= 1;
-    const double need = items / (take * kF32rWarps) + 1.0;
-    const long long blocks = need < (double)most ? (long long)need : most;
-    kern<<<(unsigned)blocks, 32 * kF32rWarps, 0, ix->stream>>>(p, take);
+    const double need = items / (TAKE * kF32rWarps) + 1.0, most = (double)device_sm_count(ix->device) * per_sm;
+    kern<<<(unsigned)(need < most ? need : most), 32 * kF32rWarps, 0, ix->stream>>>(p);
     note_launch();
     SJ_CK(cudaGetLastError());
     return SJ_OK;
+}
+
+// Items a warp takes: as many as give every warp of the chip (8 CTAs an SM) some
+// at once, but 8 of items with few evaluations, whose warps cost more than their
+// items (atomics on the queue and the cursor).  (4-D 3,000 points, 31 evaluations
+// an item: 8 at a time 20.9 us, 1 12.5; 2-D 10,000, 2 evaluations: 8 at a time
+// 10.5 us, 2 14.8.)
+template <int DP>
+int launch_f32r_d(Index* ix, const JoinParams& p, double items, bool light) {
+    const double warps = (double)device_sm_count(ix->device) * 8 * kF32rWarps;
+    if (items > 4 * warps || (light && items >= 2048)) return launch_f32r_dt<DP, 8>(ix, p, items);
+    if (items > 2 * warps) return launch_f32r_dt<DP, 4>(ix, p, items);
+    if (items > warps) return launch_f32r_dt<DP, 2>(ix, p, items);
+    return launch_f32r_dt<DP, 1>(ix, p, items);
 }
 
 }  // namespace
@@ -230,15 +241,16 @@ int launch_f32r_d(Index* ix, const JoinParams& p, double items) {
 // points) so that none is slower than k_join_f32s by more than 4%; tile us,
 // k_join_f32s / this kernel alone / shared.
 // Evenly filled cells (a point's own cell holds at most 1.4 times the mean
-// cell), this kernel alone.  Padded d <= 4: q < 2.5, and e < 160 from 2^16 items
+// cell; 1.6 in the plane from 2^17 items on: clusters 1,000,000, ratio 1.57, 867 /
+// 649 / 685), this kernel alone.  Padded d <= 4: q < 2.5, and e < 160 from 2^16 items
 // on (uniform 4-D 1,000,000 points: q 1.3 677 / 267, q 1.7, e 102 551 / 349, q
 // 2.3, e 207 460 / 423; 3-D 300,000, q 4.1 89 / 142), else e < 60 (4-D 3,000, e 31
 // 14.8 / 12.5; 1,000, e 85 13.2 / 14.5).  Padded d = 8: q < 1.9, and e < 250 from
 // 2^17 items on (5-D 1,000,000: e 99 1187 / 639; 6-D, q 1.8, e 732 1771 / 1947),
 // else e < 60 (6-D 10,000: e 77 29 / 24, e 185 34 / 41).
 // Other cells, the items of up to 3 queries, where there are enough of them for
-// two launches: 2^17 items, q < 2.5, e < 400 (clusters over noise, 3-D 342,000
-// items 520 / 1120 / 472, 4-D 511,000 588 / 606 / 432, 134,000 183 / 330 / 180,
+// two launches: 2^17 items, q < 2.5, e < 600, for d = 8 400 (clusters over noise,
+// 3-D 342,000 items 520 / 1120 / 472, 4-D 511,000 588 / 606 / 432, 134,000 183 / 330 / 180,
 // 49,000 76 / 162 / 93, 3-D 811 17 / 25 / 28).  (Batched joins and the filter's
 // recording mode keep k_join_f32s.)
 static double f32r_items(const Index* ix, double share) { return ((double)ix->n_cells + (double)ix->n / kQMax) * share; }
@@ -247,19 +259,21 @@ SparseUse f32r_use(const Index* ix, const JoinParams& p, double share) {
     if (p.batch || p.dbg || ix->n_cells <= 0) return SparseUse::none;
     const double n = (double)ix->n, cells = (double)ix->n_cells, items = f32r_items(ix, share);
     const double q = n / f32r_items(ix, 1.0), e = (double)ix->n_evaluated / f32r_items(ix, 1.0);
-    if ((double)ix->sum_sq / n > 1.4 * n / cells)
-        return items >= (1 << 17) && q < 2.5 && e < 400.0 ? SparseUse::few_queries : SparseUse::none;
+    const bool large = items >= (1 << 17);
+    if ((double)ix->sum_sq / n > (ix->dp == 2 && large ? 1.6 : 1.4) * n / cells)
+        return large && q < 2.5 && e < (ix->dp <= 4 ? 600.0 : 400.0) ? SparseUse::few_queries : SparseUse::none;
     const bool take = ix->dp <= 4 ? q < 2.5 && e < (items >= (1 << 16) ? 160.0 : 60.0)
-                                  : q < 1.9 && e < (items >= (1 << 17) ? 250.0 : 60.0);
+                                  : q < 1.9 && e < (large ? 250.0 : 60.0);
     return take ? SparseUse::all : SparseUse::none;
 }
 
 int launch_join_f32r(Index* ix, const JoinParams& p, double share) {
     const double items = f32r_items(ix, share);
+    const bool light = (double)ix->n_evaluated < 8.0 * f32r_items(ix, 1.0);
     switch (ix->dp) {
-        case 2: return launch_f32r_d<2>(ix, p, items);
-        case 4: return launch_f32r_d<4>(ix, p, items);
-        case 8: return launch_f32r_d<8>(ix, p, items);
+        case 2: return launch_f32r_d<2>(ix, p, items, light);
+        case 4: return launch_f32r_d<4>(ix, p, items, light);
+        case 8: return launch_f32r_d<8>(ix, p, items, light);
         default:
             set_error("no small-d FP32 kernel for padded dimension %d", ix->dp);
             return SJ_ERR_UNSUPPORTED;

@@ -146,8 +146,8 @@ struct KnnSplit {
     const int32_t* idx;
     const double* dist;
     __device__ __forceinline__ int4 operator[](uint32_t s) const {
-        const long long d = __double_as_longlong(__ldg(dist + s));
-        return make_int4((int)d, (int)(d >> 32), __ldg(idx + s), 0);
+        const long long d = __double_as_longlong(dist[s]);
+        return make_int4((int)d, (int)(d >> 32), idx[s], 0);
     }
 };
 
