@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(NW * 32, cc_min_blocks<T, DP, PRUNE>()) k_join
 // than 140 candidates, so that it saves whole chunks (of 128 candidates in FP64,
 // 64 in FP32) and not slots of one, and in FP64 more than 300 evaluations, for
 // its own cost an item; in FP64 with few items, which leave the chip waiting for
-// single ones, above 90 (30,000 x 3-D, 97 candidates: 67.8 / 63.8).  Planar cells
+// single ones, above 90 (30,000 x 3-D, 110 candidates: 67.8 / 63.8).  Planar cells
 // keep 83% of their candidates, so padded d = 2 goes without it in FP64 and above
 // 70 candidates with it in FP32; joins without an index go without (the box of 16
 // arbitrary points spans everything), and batches (no radius per instance for the
